@@ -515,49 +515,139 @@ __global__ void adam_kernel(float* __restrict__ P, const float* __restrict__ G, 
 // features: the state at the 27 points {-1, 0, 1}^3 of every element
 __constant__ double c_fw[kMaxN + 1][3][kMaxN + 1];   // h_m at -1, 0, 1
 
-__global__ void mlp_features_kernel(const double* __restrict__ q, const int* __restrict__ hmap,
-                                    const int* __restrict__ hang_h, const double* __restrict__ hang_w,
-                                    const int* __restrict__ col_level, int N, int nz, int NZ,
-                                    long long NG, int ncol, float s0, float s1, float s2, float s3,
-                                    float s4, float* __restrict__ F) {
-  const int n1 = N + 1, Nq = n1 * n1;
-  const long long total = (long long)ncol * nz * 27;
-  for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-       idx += (long long)gridDim.x * blockDim.x) {
-    const int pnt = (int)(idx % 27);
-    const long long e = idx / 27;
-    const int col = (int)(e / nz), k = (int)(e % nz);
-    const int pa = pnt % 3, pb = (pnt / 3) % 3, pc = pnt / 9;
-    double acc[kFields] = {0, 0, 0, 0, 0};
-    for (int c = 0; c < n1; ++c) {
-      const double wc = c_fw[N][pc][c];
-      if (wc == 0.0) continue;
+// v / s rounded to float32, for a float64 v and a float32 s, on the float32
+// and integer pipes (a float64 division per value kept the float64 pipe 87 %
+// busy): with the significands m = hi + lo of v (hi its leading 24 bits, lo
+// the next 29 rounded to float32) and t of s, one residual correction of the
+// quotient, q = q0 + (hi - q0 t + lo) / t with the residual exact in an FMA
+// (Markstein), then the exponents.  The correction is below one unit in the
+// last place of q0, so the last addition rounds the quotient to within
+// 0.5 (1 + 2^-20) units.  Quotients below half of float32's smallest value
+// give a signed zero; other results outside 2^-110 .. 2^120, infinities and
+// NaN take the float64 division.
+struct Divisor {
+  float s, t, rt;   // s, its significand with s's sign in 1 <= |t| < 2, 1 / t
+  int e;            // exponent of s; beyond the table's range for a special s
+};
+__device__ __forceinline__ Divisor divisor(float s) {
+  const unsigned b = __float_as_uint(s);
+  const int eb = (int)((b >> 23) & 0xffu);
+  Divisor d;
+  d.s = s;
+  d.t = __uint_as_float((b & 0x807fffffu) | (127u << 23));
+  d.rt = 1.0f / d.t;
+  d.e = (eb == 0 || eb == 255) ? -(1 << 20) : eb - 127;
+  return d;
+}
+__device__ __forceinline__ float div_to_f32(double v, const Divisor& D) {
+  const unsigned vh = (unsigned)__double2hiint(v), vl = (unsigned)__double2loint(v);
+  const int e = (int)((vh >> 20) & 0x7ffu) - 1023 - D.e;   // exponent of v / s, or one above it
+  const unsigned sign = vh & 0x80000000u;
+  if (e < -153) return __uint_as_float(sign ^ (__float_as_uint(D.t) & 0x80000000u));
+  if (e < -110 || e > 120) return (float)(v / (double)D.s);
+  const float hi = __uint_as_float(sign | (127u << 23) | ((vh & 0xfffffu) << 3) | (vl >> 29));
+  const float lo = __uint_as_float(__float_as_uint((float)(vl & 0x1fffffffu) * 0x1p-52f) | sign);
+  const float q0 = hi * D.rt;
+  const float q = fmaf(fmaf(-q0, D.t, hi) + lo, D.rt, q0);
+  return q * __uint_as_float((unsigned)(e + 127) << 23);
+}
+
+// Features of a column's layers [k0, k0 + KL): one CTA.  First the values of
+// the 9 horizontal points at every level that a point needs (even N: nodes
+// (a, b) in {0, N/2, N}^2 and every N/2-th level; odd N: horizontal
+// interpolation in float64 at every level), the lanes running along a
+// z-line, so the loads are contiguous; then the rows, written in the order in
+// which they lie in memory.  Bound by DRAM (the sampled lines and the 544 B
+// rows); the sampled values of neighbouring layers are formed once.  64x64x16,
+// N = 4: 30 us; 1071 us as one thread per point (27 scattered loads per element,
+// 64-bit index arithmetic, a float64 division per value).
+template <int N>
+__global__ void __launch_bounds__(256)
+mlp_features_kernel(const double* __restrict__ q, const int* __restrict__ hmap,
+                    const int* __restrict__ hang_h, const double* __restrict__ hang_w,
+                    const int* __restrict__ col_level, int nz, int NZ, long long NG, int KL, float s0,
+                    float s1, float s2, float s3, float s4, float* __restrict__ F) {
+  constexpr int n1 = N + 1, Nq = n1 * n1;
+  constexpr bool EVEN = N % 2 == 0;
+  constexpr int ST = EVEN ? N / 2 : 1;      // level stride of the staged values
+  extern __shared__ __align__(16) unsigned char smf[];
+  const int col = blockIdx.x;
+  const int LD = KL * (N / ST) + 1;         // staged level stride of (field, point)
+  float* sv = reinterpret_cast<float*>(smf);            // even N: [5][9][LD] scaled values
+  double* sd = reinterpret_cast<double*>(smf);          // odd N: [5][9][LD] values
+  const float sc[kFields] = {s0, s1, s2, s3, s4};
+  Divisor dv[kFields];
+#pragma unroll
+  for (int f = 0; f < kFields; ++f) dv[f] = divisor(sc[f]);
+  auto line = [&](int ab, int kz, double (&v)[kFields]) {
+    const int hm = hmap[(long long)col * Nq + ab];
+    if (hm >= 0) {
+      const double* p = q + (long long)hm * NZ + kz;
+#pragma unroll
+      for (int f = 0; f < kFields; ++f) v[f] = __ldg(p + f * NG);
+    } else {
+      const int hk = -1 - hm;
+#pragma unroll
+      for (int f = 0; f < kFields; ++f) v[f] = 0.0;
+      for (int m = 0; m < n1; ++m) {
+        const double w = hang_w[hk * n1 + m];
+        const double* p = q + (long long)hang_h[hk * n1 + m] * NZ + kz;
+#pragma unroll
+        for (int f = 0; f < kFields; ++f) v[f] += w * __ldg(p + f * NG);
+      }
+    }
+  };
+  for (int k0 = blockIdx.y * KL; k0 < nz; k0 += gridDim.y * KL) {
+  const int kl = min(KL, nz - k0), nlev = kl * (N / ST) + 1;
+  for (int it = threadIdx.x; it < 9 * nlev; it += blockDim.x) {
+    const int pt = it / nlev, lv = it - pt * nlev, kz = k0 * N + lv * ST;
+    const int pa = pt % 3, pb = pt / 3;
+    double v[kFields];
+    if (EVEN) {
+      line(pa * ST + n1 * (pb * ST), kz, v);
+#pragma unroll
+      for (int f = 0; f < kFields; ++f) sv[(f * 9 + pt) * LD + lv] = div_to_f32(v[f], dv[f]);
+    } else {
+      double acc[kFields] = {0, 0, 0, 0, 0};
       for (int j = 0; j < n1; ++j) {
         const double wj = c_fw[N][pb][j];
         if (wj == 0.0) continue;
         for (int i = 0; i < n1; ++i) {
           const double wi = c_fw[N][pa][i];
           if (wi == 0.0) continue;
-          const double w = wi * wj * wc;
-          const int hm = hmap[(long long)col * Nq + i + n1 * j];
-          const int kz = k * N + c;
-          if (hm >= 0) {
-            for (int f = 0; f < kFields; ++f) acc[f] += w * q[(long long)f * NG + (long long)hm * NZ + kz];
-          } else {
-            const int hk = -1 - hm;
-            for (int mm = 0; mm < n1; ++mm) {
-              const double ww = w * hang_w[hk * n1 + mm];
-              const long long o = (long long)hang_h[hk * n1 + mm] * NZ + kz;
-              for (int f = 0; f < kFields; ++f) acc[f] += ww * q[(long long)f * NG + o];
-            }
-          }
+          line(i + n1 * j, kz, v);
+#pragma unroll
+          for (int f = 0; f < kFields; ++f) acc[f] += wi * wj * v[f];
         }
       }
+#pragma unroll
+      for (int f = 0; f < kFields; ++f) sd[(f * 9 + pt) * LD + lv] = acc[f];
     }
-    const float sc[kFields] = {s0, s1, s2, s3, s4};
-    float* row = F + e * IN;
-    for (int f = 0; f < kFields; ++f) row[f * 27 + pnt] = (float)(acc[f] / sc[f]);
-    if (pnt == 0) row[135] = (float)col_level[col];
+  }
+  __syncthreads();
+  const float level = (float)col_level[col];
+  float* out = F + ((long long)col * nz + k0) * IN;
+  for (int i = threadIdx.x; i < kl * IN; i += blockDim.x) {
+    const int k = i / IN, j = i - k * IN;
+    float r = level;
+    if (j < IN - 1) {
+      const int f = j / 27, pnt = j - f * 27, pc = pnt / 9, pt = pnt - 9 * pc;
+      const int at = (f * 9 + pt) * LD;
+      if (EVEN) {
+        r = sv[at + 2 * k + pc];
+      } else {
+        double a = 0.0;
+        if (pc != 1) {
+          a = sd[at + k * N + (pc == 0 ? 0 : N)];
+        } else {
+          for (int c = 0; c < n1; ++c) a += c_fw[N][1][c] * sd[at + k * N + c];
+        }
+        r = div_to_f32(a, divisor(f == 0 ? s0 : (f == 1 ? s1 : (f == 2 ? s2 : (f == 3 ? s3 : s4)))));
+      }
+    }
+    out[i] = r;
+  }
+  __syncthreads();   // the next chunk overwrites the staged values
   }
 }
 
@@ -802,12 +892,30 @@ int mlp_features_api(Mesh& mesh, const double* q, const float* scales, float* F,
   });
   if (rc) return rc;
   DeviceTables& D = *mesh.dev;
-  const long long total = mesh.Ne() * 27;
-  const int blocks = (int)std::min<long long>((total + 255) / 256, 152 * 16);
+  // layers per CTA: 16 (a 16-layer column of the benchmark per CTA); 4 when
+  // that leaves fewer than two CTAs per SM
+  int dev = 0, nsm = 152;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  const long long ncol = mesh.Ncol();
+  int KL = std::min(16, mesh.nz);
+  if (ncol * ((mesh.nz + KL - 1) / KL) < 2LL * nsm) KL = std::min(4, mesh.nz);
+  const int chunks = (mesh.nz + KL - 1) / KL;
+  const dim3 grid((unsigned)ncol, (unsigned)std::min(chunks, 65535));
   ProfScope ps("mlp_features", st);
-  mlp_features_kernel<<<blocks, 256, 0, st>>>(q, D.hmap, D.hang_h, D.hang_w, D.col_level, mesh.N, mesh.nz,
-                                              mesh.NZ, mesh.NG, (int)mesh.Ncol(), scales[0], scales[1],
-                                              scales[2], scales[3], scales[4], F);
+  auto go = [&](auto kern, int N) {
+    const size_t sm = N % 2 == 0 ? sizeof(float) * 45 * (2 * KL + 1) : sizeof(double) * 45 * (N * KL + 1);
+    kern<<<grid, 256, sm, st>>>(q, D.hmap, D.hang_h, D.hang_w, D.col_level, mesh.nz, mesh.NZ, mesh.NG, KL,
+                                scales[0], scales[1], scales[2], scales[3], scales[4], F);
+  };
+  switch (mesh.N) {
+    case 2: go(mlp_features_kernel<2>, 2); break;
+    case 3: go(mlp_features_kernel<3>, 3); break;
+    case 4: go(mlp_features_kernel<4>, 4); break;
+    case 5: go(mlp_features_kernel<5>, 5); break;
+    case 6: go(mlp_features_kernel<6>, 6); break;
+    default: return fail(SEM_ERR_UNSUPPORTED, "order N not compiled");
+  }
   SEM_CUDA_TRY(cudaGetLastError());
   return SEM_OK;
 }
