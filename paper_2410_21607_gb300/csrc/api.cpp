@@ -128,7 +128,7 @@ int ensure_device(Mesh& m) {
   if (e == cudaSuccess) e = cudaMalloc((void**)&D.ref32, (size_t)m.NZ * (kRef + 4) * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc((void**)&D.elem_cmax, (size_t)m.Ne() * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc((void**)&D.elem_flags, (size_t)m.Ne());
-  if (e == cudaSuccess) e = cudaMalloc((void**)&D.diag_buf, (size_t)m.NZ * 4 * sizeof(double));
+  if (e == cudaSuccess) e = cudaMalloc((void**)&D.diag_buf, diag_doubles(m) * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc((void**)&D.mirror, (size_t)m.NG * kFields * sizeof(float));
   if (e != cudaSuccess) {
     free_device(m);

@@ -8,10 +8,11 @@
 //       -1 if max C^lvl <= threshold(lvl) and lvl > 0, else 0,
 //     with C^l the variable chosen for level l (speed by default; vertical
 //     vorticity or dry Ertel potential vorticity from element-local
-//     derivatives).  The speed is evaluated with explicitly rounded float64
+//     derivatives).  adapt_speed<N, EQ> is the same criterion where every level
+//     uses the speed.  The speed is evaluated with explicitly rounded float64
 //     operations (sqrt(U U + V V + W W) / rho in that order, no contraction
 //     into FMA) so that the decision is taken in float64 exactly as written.
-//   diag_level: Sec. 4.2 diagnostics, one CTA per vertical level: maximum
+//   diag_partial, diag_level: Sec. 4.2 diagnostics per vertical level: maximum
 //     horizontal speed and the mass-weighted mean speed over the horizontal
 //     sub-domain |x|, |y| <= half_width, reduced in a fixed order.
 #include <algorithm>
@@ -189,10 +190,285 @@ adapt_column(const AdaptArgs A) {
   }
 }
 
+
+// The speed criterion (no derivatives).  What it needs per element is the
+// maximum over the nodes of s = sqrt(U U + V V + W W) / rho in float64, and
+// a float64 square root and divide at every node is what the general kernel
+// above spends its time on (float64 pipe; 64x64x16, N = 4: 672 us for 137 MB of
+// state, here 59 us).  Here a thread owns a level of a column and first bounds s at the
+// level's (N+1)^2 nodes in float32; only nodes whose upper bound reaches the
+// largest lower bound of a layer they belong to can hold its maximum, and
+// only those are evaluated in float64, with the same rounded operations in
+// the same order, so the maxima and the flags are those of the general kernel
+// bit for bit.  A layer whose bounds are of no use (a density that is not
+// positive, values outside float32's range, a tiny maximum) evaluates all of
+// its nodes; a plane of exact zeros has the maximum 0.  A level that two
+// layers share is bounded once.  Lanes run along z, so the loads are
+// contiguous; what is left is instruction issue and the loads' latency.
+template <int N, int EQ>
+__device__ __forceinline__ void criterion_node(const AdaptArgs& A, const int hm, const int kz, double (&v)[4]) {
+  // rho', U, V, W as the general kernel forms them
+  if (hm >= 0) {
+    const double* p = A.q + (long long)hm * A.NZ + kz;
+#pragma unroll
+    for (int f = EQ == 0 ? 0 : 1; f < 4; ++f) v[f] = __ldg(p + (long long)f * A.NG);
+  } else {
+    const int h = -1 - hm;
+#pragma unroll
+    for (int f = 0; f < 4; ++f) v[f] = 0.0;
+    for (int m = 0; m <= N; ++m) {
+      const double w = A.hang_w[h * (N + 1) + m];
+      const double* p = A.q + (long long)A.hang_h[h * (N + 1) + m] * A.NZ + kz;
+#pragma unroll
+      for (int f = EQ == 0 ? 0 : 1; f < 4; ++f) v[f] = __dadd_rn(v[f], __dmul_rn(w, __ldg(p + (long long)f * A.NG)));
+    }
+  }
+}
+__device__ __forceinline__ double ref_rho(const AdaptArgs& A, const int hm, const int kz) {
+  const double* rf = !A.refG ? A.ref + (long long)kz * kRef
+                     : (hm >= 0 ? A.refG + ((long long)hm * A.NZ + kz) * kRef
+                                : A.refH + ((long long)(-1 - hm) * A.NZ + kz) * kRef);
+  return rf[3];
+}
+template <int N, int EQ>
+__device__ __noinline__ double exact_speed(const AdaptArgs& A, const int hm, const int kz) {
+  double v[4];
+  criterion_node<N, EQ>(A, hm, kz, v);
+  const double ss = __dadd_rn(__dadd_rn(__dmul_rn(v[1], v[1]), __dmul_rn(v[2], v[2])), __dmul_rn(v[3], v[3]));
+  double s = __dsqrt_rn(ss);
+  if (EQ == 0) s = __ddiv_rn(s, __dadd_rn(ref_rho(A, hm, kz), v[0]));
+  return s;
+}
+// |x| as float32 by its bits (significand truncated).  Values below 2^-100
+// give 0; `u` is the magnitude's upper half, for the caller's range checks.
+constexpr unsigned kTinyHi = (1023u - 100u) << 20, kHugeHi = (1023u + 100u) << 20, kZeroHi = (1023u - 540u) << 20;
+__device__ __forceinline__ float mag_f32(double x, unsigned& u) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  u = hi & 0x7fffffffu;
+  // the 11-bit exponent less 896 is its low 8 bits with the top one flipped
+  const float f = __uint_as_float((__funnelshift_l(lo, hi, 3) & 0x7fffffffu) ^ 0x40000000u);
+  return u < kTinyHi ? 0.f : f;
+}
+__device__ __forceinline__ float near_f32(double x, unsigned& u) {
+  return copysignf(mag_f32(x, u), __int_as_float(__double2hiint(x)));
+}
+// What a thread collects over its plane: ranges of the magnitudes' upper
+// halves and of the density, from which the plane's bounds are judged once.
+struct PlaneRange {
+  unsigned top = 0u, low = 0u;   // largest magnitude; largest one that counted as 0
+  float rmin = 1e30f, rmax = -1e30f;
+};
+// s^2 at a node in float32 and the factor-free excess e by which a hanging
+// node's s may be larger.  Every operand is within 2^-23 of its value, the
+// density (checked to stay within 1/4 .. 4 of its reference) within 7 2^-23,
+// and the products, sums and the reciprocal add a few units: s^2 is within
+// 6e-6 of its value, for which kSlack = 1e-5 is taken.  A hanging node is a
+// weighted sum of nodes: its terms are bounded by their absolute sums.
+constexpr float kSlack = 1e-5f;
+template <int N, int EQ>
+__device__ __forceinline__ float speed2(const AdaptArgs& A, const int hm, const int kz, const float rho0,
+                                        PlaneRange& R, float& e) {
+  float r = 1.f, s2;
+  unsigned u;
+  e = 0.f;
+  if (hm >= 0) {
+    const double* p = A.q + (long long)hm * A.NZ + kz;
+    double d[4];
+#pragma unroll
+    for (int f = EQ == 0 ? 0 : 1; f < 4; ++f) d[f] = __ldg(p + (long long)f * A.NG);
+    if (EQ == 0) {
+      r = rho0 + near_f32(d[0], u);
+      R.top = max(R.top, u);
+    }
+    s2 = 0.f;
+#pragma unroll
+    for (int f = 1; f < 4; ++f) {
+      const float x = mag_f32(d[f], u);
+      R.top = max(R.top, u);
+      R.low = max(R.low, u < kTinyHi ? u : 0u);
+      s2 = fmaf(x, x, s2);
+    }
+  } else {
+    const int h = -1 - hm;
+    float x[3] = {0.f, 0.f, 0.f}, a = 0.f, ar = 0.f;
+    r = EQ == 0 ? 0.f : 1.f;
+    for (int m = 0; m <= N; ++m) {
+      const float w = near_f32(A.hang_w[h * (N + 1) + m], u);
+      const double* p = A.q + (long long)A.hang_h[h * (N + 1) + m] * A.NZ + kz;
+#pragma unroll
+      for (int f = 0; f < 3; ++f) {
+        const float t = w * near_f32(__ldg(p + (long long)(f + 1) * A.NG), u);
+        R.top = max(R.top, u);
+        R.low = max(R.low, u < kTinyHi ? u : 0u);
+        x[f] += t;
+        a += fabsf(t);
+      }
+      if (EQ == 0) {
+        const float t = w * near_f32(__ldg(p), u);
+        R.top = max(R.top, u);
+        r += t;
+        ar += fabsf(t);
+      }
+    }
+    if (EQ == 0) r += rho0;
+    // a density that is too uncertain for the bounds: none
+    if (EQ == 0 && !(ar * 4e-6f < 1e-7f * r)) r = -1.f;
+    e = __fdividef(4e-6f * a, r);
+    s2 = fmaf(x[0], x[0], fmaf(x[1], x[1], x[2] * x[2]));
+  }
+  if (EQ == 0) {
+    R.rmin = fminf(R.rmin, r);
+    R.rmax = fmaxf(R.rmax, r);
+    const float inv = __fdividef(1.f, r);
+    s2 *= inv * inv;
+  }
+  return s2;
+}
+// the upper bound on s^2 from it
+__device__ __forceinline__ float upper2(float s2, float e) {
+  if (e > 0.f) {
+    const float s = sqrtf(s2) + e;
+    s2 = s * s;
+  }
+  return s2 * (1.f + kSlack);
+}
+
+constexpr int kSpeedThreads = 256;
+template <int N, int EQ>
+__global__ void __launch_bounds__(kSpeedThreads)
+adapt_speed(const AdaptArgs A, const int ncol, const int cols, const int KL) {
+  constexpr int n1 = N + 1, Nq = n1 * n1;
+  extern __shared__ double s_ex[];                      // [items] exact maximum of a level, NaN: not needed
+  const int LV = KL * N + 1;                            // levels of a chunk of KL layers
+  float* s_lo = reinterpret_cast<float*>(s_ex + cols * LV);   // [items] largest lower bound on s^2
+  float* s_hi = s_lo + cols * LV;                       // [items] largest upper bound; infinity: none
+  for (int k0 = blockIdx.y * KL; k0 < A.nz; k0 += gridDim.y * KL) {
+    const int kl = min(KL, A.nz - k0), nlev = kl * N + 1;
+    const int c0 = blockIdx.x * cols, nc = min(cols, ncol - c0), items = nc * nlev;
+    const int t = threadIdx.x;
+    const bool act = t < items;
+    const int lc = act ? t / nlev : 0, lv = act ? t - lc * nlev : 0, kz = k0 * N + lv;
+    const int* hmap = A.hmap + (long long)(c0 + lc) * Nq;
+    float lo = 0.f, hi = 0.f, hi2 = 0.f;
+    int arg = 0;
+    const float inf = __int_as_float(0x7f800000);
+    if (act) {
+      const float rho0 = EQ == 0 ? (float)A.ref[(long long)kz * kRef + 3] : 1.f;
+      PlaneRange R;
+      bool fits = rho0 > 1e-6f && rho0 < 1e20f;
+#pragma unroll 5
+      for (int ab = 0; ab < Nq; ++ab) {
+        const int hm = hmap[ab];
+        float r0 = rho0, e;
+        if (EQ == 0 && A.refG) {
+          // warped layers: the node's own reference density, taken relative to rho0's range
+          r0 = (float)ref_rho(A, hm, kz);
+          fits = fits && r0 > 0.5f * rho0 && r0 < 2.f * rho0;
+        }
+        const float s2 = speed2<N, EQ>(A, hm, kz, r0, R, e), u2 = upper2(s2, e);
+        if (e == 0.f) lo = fmaxf(lo, s2);
+        if (u2 > hi) {
+          hi2 = hi;
+          hi = u2;
+          arg = ab;
+        } else {
+          hi2 = fmaxf(hi2, u2);
+        }
+      }
+      lo *= 1.f - kSlack;
+      // a plane whose bounds say nothing: infinity
+      if (EQ == 0) fits = fits && R.rmin > 0.5f * rho0 && R.rmax < 2.f * rho0;
+      fits = fits && R.top < kHugeHi && hi < 1e34f && !(R.low > kZeroHi && hi < 1e-24f);
+      s_lo[t] = lo;
+      s_hi[t] = fits ? hi : inf;
+    }
+    __syncthreads();
+    if (act) {
+      // the smaller of the layers' lower bounds that this level has to reach;
+      // -1 (every node) where a layer holds a plane without bounds
+      float need = inf;
+      for (int s = 0; s < 2; ++s) {
+        const int k = lv / N - s;                      // layers [k N, k N + N] that hold the level
+        if (k < 0 || k >= kl || lv > k * N + N) continue;
+        float m = 0.f, h = 0.f;
+        for (int c = 0; c <= N; ++c) {
+          m = fmaxf(m, s_lo[lc * nlev + k * N + c]);
+          h = fmaxf(h, s_hi[lc * nlev + k * N + c]);
+        }
+        // a maximum below 1e-12 (s^2 below 1e-24): squares near float32's
+        // underflow, no bound, except planes of zeros (hi = 0)
+        if (!(h < 1e34f) || (h > 0.f && m < 1e-24f)) m = -1.f;
+        need = fminf(need, m);
+      }
+      double ex = __longlong_as_double(0x7ff8000000000000ll);   // fmax ignores it
+      if (need < 0.f || hi2 >= need) {
+        if (need == 0.f && hi == 0.f) {
+          ex = 0.0;                                    // zeros throughout
+        } else {
+          for (int ab = 0; ab < Nq; ++ab) {
+            const int hm = hmap[ab];
+            if (need >= 0.f) {
+              PlaneRange R;
+              float e;
+              const float s2 = speed2<N, EQ>(A, hm, kz, EQ == 0 ? (float)ref_rho(A, hm, kz) : 1.f, R, e);
+              if (upper2(s2, e) < need) continue;
+            }
+            ex = fmax(ex, exact_speed<N, EQ>(A, hm, kz));
+          }
+        }
+      } else if (hi >= need) {
+        ex = exact_speed<N, EQ>(A, hmap[arg], kz);
+      }
+      s_ex[t] = ex;
+    }
+    __syncthreads();
+    for (int el = t; el < nc * kl; el += blockDim.x) {
+      const int c = el / kl, k = el - c * kl;
+      double mx = s_ex[c * nlev + k * N];
+      for (int i = 1; i <= N; ++i) mx = fmax(mx, s_ex[c * nlev + k * N + i]);
+      // the general kernel's idle lanes hold 0
+      if ((n1 * Nq) % 32 != 0) mx = fmax(mx, 0.0);
+      const long long e = (long long)(c0 + c) * A.nz + k0 + k;
+      const int lev = A.elem_level ? (int)A.elem_level[e] : (A.level_all >= 0 ? A.level_all : A.col_level[c0 + c]);
+      int flag = 0;
+      if (lev < A.lvl_max && mx > A.thr[lev]) flag = 1;
+      else if (lev > 0 && mx <= A.thr[lev - 1]) flag = -1;
+      A.flags[e] = (int8_t)flag;
+      if (A.cmax) A.cmax[e] = mx;
+    }
+    __syncthreads();
+  }
+}
+
+template <int N>
+static void launch_speed(const AdaptArgs& A, int ncol, int eq, cudaStream_t st) {
+  // layers per chunk: as many as the block's threads have levels; columns per
+  // block: as many as fill it, one where the mesh has too few of them to give
+  // every SM two blocks
+  int dev = 0, nsm = 152;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  const int KL = std::min(A.nz, (kSpeedThreads - 1) / N), LV = KL * N + 1;
+  const int chunks = (A.nz + KL - 1) / KL;
+  int cols = kSpeedThreads / LV;
+  while (cols > 1 && (long long)((ncol + cols - 1) / cols) * chunks < 2LL * nsm) --cols;
+  const int nt = (cols * LV + 31) / 32 * 32;
+  const dim3 grid((unsigned)((ncol + cols - 1) / cols), (unsigned)std::min(chunks, 65535));
+  const size_t sm = (size_t)cols * LV * 16;
+  if (eq == 0)
+    adapt_speed<N, 0><<<grid, nt, sm, st>>>(A, ncol, cols, KL);
+  else
+    adapt_speed<N, 1><<<grid, nt, sm, st>>>(A, ncol, cols, KL);
+}
+
 template <int N>
 static void launch_adapt_n(const AdaptArgs& A, int ncol, int eq, cudaStream_t st) {
   constexpr int P = (N + 1) * (N + 1) * (N + 1);
   constexpr int nt = (P + 31) / 32 * 32;
+  // the speed at every level: bounded in float32 first
+  bool speed = true;
+  for (int k = 0; k < SEM_MAX_THRESHOLDS; ++k) speed = speed && A.var[k] == SEM_CRIT_SPEED;
+  if (speed) return launch_speed<N>(A, ncol, eq, st);
   if (eq == 0)
     adapt_column<N, 0><<<ncol, nt, 0, st>>>(A);
   else
@@ -252,26 +528,82 @@ int launch_adapt(Mesh& m, const sem_params& p, const double* q, int8_t* flags, d
 }
 
 // ---------------------------------------------------------------------------
+// Wind diagnostics in two passes.  diag_partial: one CTA per 32 horizontal
+// nodes lists those inside the sub-domain (most CTAs have none and end there)
+// and, lanes along z so that the loads are contiguous, reduces each level over
+// the list, dealt out to as many groups of warps as fit (a node costs a float64
+// root and a divide, in a serial chain per level), the groups' values added in
+// order; diag_level: one CTA per level reduces the CTAs' partial values in a
+// fixed order.  64x64x16, N = 4, 100 km: 28 + 7 us; 135 us as one CTA per level
+// walking all horizontal nodes with loads NZ apart.
+constexpr int kDiagLines = 32, kDiagThreads = 384;
+__global__ void __launch_bounds__(kDiagThreads)
+diag_partial(const double* __restrict__ q, const double* __restrict__ xh, const double* __restrict__ yh,
+             const double* __restrict__ Mh, const double* __restrict__ ref, long long NH, int NZ, long long NG,
+             double hw, int eq, const double* __restrict__ refG, const double* __restrict__ Minv_g,
+             double* __restrict__ part /*[chunks][NZ][3]*/, int* __restrict__ count) {
+  __shared__ int s_h[kDiagLines];
+  const long long h0 = (long long)blockIdx.x * kDiagLines;
+  const int lane = threadIdx.x & 31;
+  const bool in = h0 + lane < NH && fabs(xh[h0 + lane]) <= hw + 1e-6 && fabs(yh[h0 + lane]) <= hw + 1e-6;
+  const unsigned mask = __ballot_sync(0xffffffffu, in);
+  const int n = __popc(mask);
+  if (threadIdx.x == 0) count[blockIdx.x] = n;
+  if (n == 0) return;
+  if (threadIdx.x < 32 && in) s_h[__popc(mask & ((1u << lane) - 1u))] = lane;
+  __shared__ double s_v[3][kDiagThreads];
+  const int LVT = min((NZ + 31) & ~31, kDiagThreads);   // threads of a group: one per level
+  const int groups = kDiagThreads / LVT, gr = threadIdx.x / LVT, lt = threadIdx.x - gr * LVT;
+  for (int k0 = 0; k0 < NZ; k0 += LVT) {
+    __syncthreads();
+    const int kz = k0 + lt;
+    double mx = 0.0, num = 0.0, den = 0.0;
+    if (kz < NZ && gr < groups) {
+      const double rho0 = ref[(long long)kz * kRef + 3];
+#pragma unroll 2
+      for (int i = gr; i < n; i += groups) {
+        const long long h = h0 + s_h[i], g = h * NZ + kz;
+        const double U = q[NG + g], V = q[2 * NG + g];
+        double s = sqrt(U * U + V * V);
+        // warped layers: the node's own reference density and lumped mass (the
+        // level means are then over a grid level, not a height)
+        if (eq == 0) s = s / ((refG ? refG[g * kRef + 3] : rho0) + q[g]);
+        const double wm = Minv_g ? 1.0 / Minv_g[g] : Mh[h];
+        mx = fmax(mx, s);
+        num += wm * s;
+        den += wm;
+      }
+    }
+    s_v[0][threadIdx.x] = mx;
+    s_v[1][threadIdx.x] = num;
+    s_v[2][threadIdx.x] = den;
+    __syncthreads();
+    if (gr == 0 && kz < NZ) {
+      for (int i = 1; i < groups; ++i) {
+        mx = fmax(mx, s_v[0][i * LVT + lt]);
+        num += s_v[1][i * LVT + lt];
+        den += s_v[2][i * LVT + lt];
+      }
+      double* o = part + ((long long)blockIdx.x * NZ + kz) * 3;
+      o[0] = mx;
+      o[1] = num;
+      o[2] = den;
+    }
+  }
+}
+
 __global__ void __launch_bounds__(256)
-diag_level(const double* q, const double* xh, const double* yh, const double* Mh,
-           const double* ref, long long NH, int NZ, long long NG, double hw, int eq,
-           const double* refG, const double* Minv_g, double* out /*[NZ][4]*/) {
+diag_level(const double* __restrict__ part, const int* __restrict__ count, int chunks, int NZ,
+           double* __restrict__ out /*[NZ][4]*/) {
   __shared__ double s_max[256], s_num[256], s_den[256];
   const int kz = blockIdx.x;
-  const double rho0 = ref[(long long)kz * kRef + 3];
   double mx = 0.0, num = 0.0, den = 0.0;
-  for (long long h = threadIdx.x; h < NH; h += blockDim.x) {
-    if (!(fabs(xh[h]) <= hw + 1e-6 && fabs(yh[h]) <= hw + 1e-6)) continue;
-    const long long g = h * NZ + kz;
-    const double U = q[NG + g], V = q[2 * NG + g];
-    double s = sqrt(U * U + V * V);
-    // warped layers: the node's own reference density and lumped mass (the
-    // level means are then over a grid level, not a height)
-    if (eq == 0) s = s / ((refG ? refG[g * kRef + 3] : rho0) + q[g]);
-    const double wm = Minv_g ? 1.0 / Minv_g[g] : Mh[h];
-    mx = fmax(mx, s);
-    num += wm * s;
-    den += wm;
+  for (int c = threadIdx.x; c < chunks; c += blockDim.x) {
+    if (count[c] == 0) continue;
+    const double* p = part + ((long long)c * NZ + kz) * 3;
+    mx = fmax(mx, p[0]);
+    num += p[1];
+    den += p[2];
   }
   s_max[threadIdx.x] = mx;
   s_num[threadIdx.x] = num;
@@ -293,12 +625,21 @@ diag_level(const double* q, const double* xh, const double* yh, const double* Mh
   }
 }
 
+// doubles of D.diag_buf: the levels' results, the partial values, the counts
+size_t diag_doubles(const Mesh& m) {
+  const size_t chunks = (size_t)((m.NH + kDiagLines - 1) / kDiagLines);
+  return (size_t)m.NZ * 4 + chunks * m.NZ * 3 + (chunks + 1) / 2;
+}
+
 int launch_diag(Mesh& m, const sem_params& p, const double* q, double hw, sem_diag_out* out,
                 cudaStream_t st) {
   DeviceTables& D = *m.dev;
-  diag_level<<<m.NZ, 256, 0, st>>>(q, D.xh, D.yh, D.Mh, D.ref, m.NH, m.NZ, m.NG, hw, p.eqset,
-                                    m.warped() ? D.refG : nullptr, m.warped() ? D.Minv_g : nullptr,
-                                    D.diag_buf);
+  const int chunks = (int)((m.NH + kDiagLines - 1) / kDiagLines);
+  double* part = D.diag_buf + (size_t)m.NZ * 4;
+  int* count = reinterpret_cast<int*>(part + (size_t)chunks * m.NZ * 3);
+  diag_partial<<<chunks, kDiagThreads, 0, st>>>(q, D.xh, D.yh, D.Mh, D.ref, m.NH, m.NZ, m.NG, hw, p.eqset,
+                                       m.warped() ? D.refG : nullptr, m.warped() ? D.Minv_g : nullptr, part, count);
+  diag_level<<<m.NZ, 256, 0, st>>>(part, count, chunks, m.NZ, D.diag_buf);
   SEM_CUDA_TRY(cudaGetLastError());
   std::vector<double> buf((size_t)m.NZ * 4);
   SEM_CUDA_TRY(cudaMemcpyAsync(buf.data(), D.diag_buf, buf.size() * sizeof(double),

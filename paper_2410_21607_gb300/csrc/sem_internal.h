@@ -181,7 +181,7 @@ struct DeviceTables {
   // adapt and diagnostics
   double* elem_cmax = nullptr;
   int8_t* elem_flags = nullptr;
-  double* diag_buf = nullptr;   // [NZ][4]
+  double* diag_buf = nullptr;   // [NZ][4], then the partial reductions (diag_doubles)
   // continuous projection of the transfer (coupled coarse-face nodes)
   int n_comp = 0, max_comp = 0;
   int* tr_comp_ptr = nullptr;   // [n_comp+1] into tr_nodes
@@ -240,6 +240,7 @@ int launch_adapt(Mesh& m, const sem_params& p, const double* q, int8_t* flags, d
                  cudaStream_t st, const int8_t* elem_level = nullptr, int level_all = -1);
 int launch_merge_flags(const int8_t* crit, const int8_t* pred, const int8_t* level, int lvl_max, long long n,
                        int8_t* out, cudaStream_t st);
+size_t diag_doubles(const Mesh& m);
 int launch_diag(Mesh& m, const sem_params& p, const double* q, double half_width,
                 sem_diag_out* out, cudaStream_t st);
 int launch_transfer(Mesh& oldm, Mesh& newm, const double* qold, double* qnew, cudaStream_t st);
