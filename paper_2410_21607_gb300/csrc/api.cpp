@@ -38,7 +38,7 @@ void free_device(Mesh& m) {
   void* ptrs[] = {D.hmap, D.hang_h, D.hang_w, D.qt_ptr, D.qt_src, D.qt_w, D.Minv_h, D.Minv_z,
                   D.Mh, D.Mz, D.Minv_h32, D.Minv_z32, D.qt_w32, D.qt_rec_src, D.qt_rec_w, D.qt_rec_unit, D.hang_w32, D.mirror, D.spg, D.spg32, D.ref, D.ref32, D.col_level, D.col_x0, D.col_y0, D.xh, D.yh, D.zk, D.hzk, D.hzk32, D.scratch,
                   D.status, D.org, D.elem_cmax, D.elem_flags, D.diag_buf,
-                  D.tr_comp_ptr, D.tr_nodes, D.tr_A_ptr, D.tr_A_col, D.tr_A_val, D.tr_coupled,
+                  D.tr_comp_ptr, D.tr_nodes, D.tr_A_ptr, D.tr_A_col, D.tr_A_val, D.tr_coupled, D.tr_A32, D.tr_S, D.tr_meta,
                   D.zG, D.zH, D.metric, D.metric32, D.Minv_g, D.Minv_g32, D.refG, D.refH, D.refG32, D.refH32,
                   D.ref4G, D.ref4H};
   for (void* p : ptrs)

@@ -11,8 +11,12 @@
 //      (Q^T W Q) q_G = Q^T W q_L with W the LGL quadrature weights times the
 //      Jacobian.  Q^T W Q = A_h (x) M_z: diagonal (the lumped mass) except on
 //      the coarse-side nodes that hanging rows couple; those small coupled
-//      blocks are solved by a Jacobi-preconditioned conjugate gradient, one
-//      CTA per (block, field, level), with a bounded iteration count.
+//      blocks are solved by float64 iterative refinement whose corrections
+//      come from a Jacobi-preconditioned float32 conjugate gradient, with
+//      bounded iteration counts.
+// The float64 pipe of this part is narrow (1/64 of the float32 rate): even a
+// weight per copied value would bound a copy, so unchanged values are moved,
+// not multiplied.
 // The projection keeps every continuous field (refinement changes nothing)
 // and the lumped total of every field.
 #include <algorithm>
@@ -23,7 +27,7 @@
 namespace sem {
 
 __constant__ double c_P[kMaxN + 1][2][(kMaxN + 1) * (kMaxN + 1)];  // child interpolation
-__constant__ double c_R[kMaxN + 1][2][(kMaxN + 1) * (kMaxN + 1)];  // child L2 projection
+__constant__ double c_R[kMaxN + 1][2][(kMaxN + 1) * (kMaxN + 1)];  // child L2 projection, halved
 __constant__ double c_tw[kMaxN + 1][kMaxN + 1];                     // LGL weights
 
 static int upload_transfer_constants_now() {
@@ -68,7 +72,7 @@ static int upload_transfer_constants_now() {
         for (int j = 0; j < n; ++j) {
           double s = 0.0;
           for (int q = 0; q < n; ++q) s += Mi[i * n + q] * T[q * n + j];
-          R[N][c][i * n + j] = s;
+          R[N][c][i * n + j] = 0.5 * s;   // with the 1/4 of the four children
           P[N][c][i * n + j] = B.P[c][i * n + j];
         }
     }
@@ -94,202 +98,386 @@ struct TrArgs {
   long long old_NG;
   const int* org;      // [Ncol][6]
   const int* new_level;
-  double* out;         // new scratch [Ncol][Nq][5][NZ]
-  int nz, NZ;
-  double Lx, Ly, Lz;
-  int nx, ny;
-  const double* hzk;   // [nz] layer thicknesses
+  double* out;         // new scratch [Ncol][Nq][5][NZ], mapped columns only
+  int N, NZ;
+  double hxy;          // Lx Ly / (nx ny) / 4: J of a level-0 column per unit w_a w_b
 };
 
+// New values of the refined and coarsened columns, out[col][ab][f][kz].  One
+// CTA per new column (those of unchanged columns end at once); a thread owns
+// one level of one field and holds the level's (N+1)^2 nodes in registers, so
+// the two directions are contracted one after the other (per node and field
+// 2 (N+1) FMAs for a refined column, 6 (N+1) for a coarsened one, where the
+// 2-D operators applied node by node take (N+1)^2 and 4 (N+1)^2 and their
+// weights), the operators are read as uniform constants and the lanes run
+// along z.  Bound by the float64 pipe.  No factor of the vertical direction
+// enters: parent and children share the levels, and the layers' weights
+// cancel against the vertical lumped mass.  Remesh of 113 k elements, N = 4:
+// 468 us, and 147 us for transfer_gather, which moves the unchanged lines
+// itself; 2348 and 204 us when every column was mapped node by node and every
+// value weighted.
 template <int N>
-__device__ __forceinline__ void gather_old(const TrArgs& A, int col, int ab, int kz, double v[kFields]) {
+__device__ __forceinline__ double old_value(const TrArgs& A, const int hm, const int f, const int kz) {
+  const double* q = A.qold + (long long)f * A.old_NG + kz;
+  if (hm >= 0) return __ldg(q + (long long)hm * A.NZ);
+  const int k = -1 - hm;
+  double v = 0.0;
+#pragma unroll
+  for (int m = 0; m <= N; ++m)
+    v += A.old_hang_w[k * (N + 1) + m] * __ldg(q + (long long)A.old_hang_h[k * (N + 1) + m] * A.NZ);
+  return v;
+}
+// One (field, level) of a new column from its source columns.  The operator
+// tables are indexed directly (not through a selected pointer, which would make
+// their loads generic), c and d being the same for the whole CTA.
+template <int N, bool COARSE>
+__device__ __forceinline__ void new_plane(const TrArgs& A, const int* o, const int f, const int kz,
+                                          double (&acc)[(N + 1) * (N + 1)]) {
   constexpr int n1 = N + 1, Nq = n1 * n1;
-  const int hm = A.old_hmap[(long long)col * Nq + ab];
-  if (hm >= 0) {
-    for (int f = 0; f < kFields; ++f) v[f] = A.qold[(long long)f * A.old_NG + (long long)hm * A.NZ + kz];
-  } else {
-    const int k = -1 - hm;
-    for (int f = 0; f < kFields; ++f) v[f] = 0.0;
-    for (int m = 0; m <= N; ++m) {
-      const double w = A.old_hang_w[k * n1 + m];
-      const long long o = (long long)A.old_hang_h[k * n1 + m] * A.NZ + kz;
-      for (int f = 0; f < kFields; ++f) v[f] += w * A.qold[(long long)f * A.old_NG + o];
+#pragma unroll
+  for (int ab = 0; ab < Nq; ++ab) acc[ab] = 0.0;
+#pragma unroll 1
+  for (int b = 0; b < (COARSE ? 2 : 1); ++b) {
+    double v[Nq];   // contracted along x
+#pragma unroll
+    for (int ab = 0; ab < Nq; ++ab) v[ab] = 0.0;
+#pragma unroll 1
+    for (int a = 0; a < (COARSE ? 2 : 1); ++a) {
+      const int ca = COARSE ? a : (o[5] & 1);
+      const int* hm = A.old_hmap + (long long)o[1 + a + 2 * b] * Nq;
+#pragma unroll
+      for (int j = 0; j < n1; ++j) {
+        double r[n1];
+#pragma unroll
+        for (int m = 0; m < n1; ++m) r[m] = old_value<N>(A, hm[m + n1 * j], f, kz);
+#pragma unroll
+        for (int i = 0; i < n1; ++i)
+#pragma unroll
+          for (int m = 0; m < n1; ++m)
+            v[i + n1 * j] = fma(COARSE ? c_R[N][ca][i * n1 + m] : c_P[N][ca][i * n1 + m], r[m], v[i + n1 * j]);
+      }
     }
+    const int cb = COARSE ? b : (o[5] >> 1);
+#pragma unroll
+    for (int j = 0; j < n1; ++j)
+#pragma unroll
+      for (int n = 0; n < n1; ++n) {
+        const double y = COARSE ? c_R[N][cb][j * n1 + n] : c_P[N][cb][j * n1 + n];
+#pragma unroll
+        for (int i = 0; i < n1; ++i) acc[i + n1 * j] = fma(y, v[i + n1 * n], acc[i + n1 * j]);
+      }
   }
 }
 
+constexpr int kTrThreads = 192;
 template <int N>
-__global__ void __launch_bounds__(((N + 1) * (N + 1) * (N + 1) + 31) / 32 * 32)
+__global__ void __launch_bounds__(kTrThreads, N <= 4 ? 2 : 1)
 transfer_local(const TrArgs A) {
-  constexpr int n1 = N + 1, Nq = n1 * n1, P = n1 * n1 * n1;
-  __shared__ double sQ[4][kFields][P];
-  __shared__ double sC[2][kFields][Nq];
-  const int col = blockIdx.x, t = threadIdx.x;
-  const bool act = t < P;
-  const int i = t % n1, j = (t / n1) % n1, c = t / Nq;
-  const int ab = i + n1 * j;
+  constexpr int Nq = (N + 1) * (N + 1);
+  const int col = blockIdx.x;
   const int* o = A.org + (long long)col * 6;
   const int kind = o[0];
-  const int lev = A.new_level[col];
-  const double hx = A.Lx / (double)((long long)A.nx << lev);
-  const double hy = A.Ly / (double)((long long)A.ny << lev);
-  const double wJ1 = act ? c_tw[N][i] * c_tw[N][j] * c_tw[N][c] * hx * hy * 0.125 : 0.0;  // per unit thickness
-  const int nsrc = kind == 2 ? 4 : 1;
-  for (int k = 0; k < A.nz; ++k) {
-    const int kz = k * N + c;
-    if (act) {
-      for (int s = 0; s < nsrc; ++s) {
-        double v[kFields];
-        gather_old<N>(A, o[1 + s], ab, kz, v);
-        for (int f = 0; f < kFields; ++f) sQ[s][f][t] = v[f];
+  if (kind == 0) return;
+  const long long ld = (long long)kFields * A.NZ;
+  for (int it = threadIdx.x; it < kFields * A.NZ; it += blockDim.x) {
+    const int f = it / A.NZ, kz = it - f * A.NZ;
+    double acc[Nq];
+    if (kind == 1) new_plane<N, false>(A, o, f, kz, acc);
+    else new_plane<N, true>(A, o, f, kz, acc);
+    double* dst = A.out + ((long long)col * Nq * kFields + f) * A.NZ + kz;
+#pragma unroll
+    for (int ab = 0; ab < Nq; ++ab) dst[ab * ld] = acc[ab];
+  }
+}
+
+// Where the new line h comes from: meta[h] >= 0: every source is an unchanged
+// column's node of the same old line, whose weighted mean is that line (a
+// copy); meta[h] <= -2: the only source is node -2 - meta[h] of a mapped
+// column; -1: the weighted sum over the sources.
+__global__ void transfer_meta(const TrArgs A, const int4* __restrict__ rec_unit, const int* __restrict__ coupled,
+                              int NH, int* __restrict__ meta) {
+  const int h = blockIdx.x * blockDim.x + threadIdx.x;
+  if (h >= NH) return;
+  const int Nq = (A.N + 1) * (A.N + 1);
+  const int4 r = rec_unit[h];
+  int m = -1;
+  if (r.x >= 0 && !coupled[h]) {
+    const int src[4] = {r.x, r.y, r.z, r.w};
+    const int* o = A.org + (long long)(r.x / Nq) * 6;
+    if (o[0] != 0) {
+      if (r.y < 0) m = -2 - r.x;
+    } else {
+      m = A.old_hmap[(long long)o[1] * Nq + r.x % Nq];
+      for (int e = 1; e < 4 && src[e] >= 0 && m >= 0; ++e) {
+        const int* oe = A.org + (long long)(src[e] / Nq) * 6;
+        if (oe[0] != 0 || A.old_hmap[(long long)oe[1] * Nq + src[e] % Nq] != m) m = -1;
       }
+      if (m < 0) m = -1;
     }
-    __syncthreads();
-    double r[kFields] = {0, 0, 0, 0, 0};
-    if (act) {
-      if (kind == 0) {
-        for (int f = 0; f < kFields; ++f) r[f] = sQ[0][f][t];
-      } else if (kind == 1) {
-        const int ca = o[5] & 1, cb = o[5] >> 1;
-        for (int m = 0; m < n1; ++m)
-          for (int n = 0; n < n1; ++n) {
-            const double w = c_P[N][ca][i * n1 + m] * c_P[N][cb][j * n1 + n];
-            for (int f = 0; f < kFields; ++f) r[f] += w * sQ[0][f][m + n1 * n + Nq * c];
+  }
+  meta[h] = m;
+}
+
+__global__ void __launch_bounds__(256)
+transfer_gather(const TrArgs A, const int* __restrict__ meta, const int* __restrict__ qt_ptr,
+                const int* __restrict__ qt_src, const double* __restrict__ qt_w,
+                const double* __restrict__ Minv_h, const int* __restrict__ coupled, unsigned NG,
+                double* __restrict__ q) {
+  const unsigned NZ = (unsigned)A.NZ;
+  for (unsigned g = blockIdx.x * blockDim.x + threadIdx.x; g < NG; g += gridDim.x * blockDim.x) {
+    const unsigned h = g / NZ, kz = g - h * NZ;
+    const int m = __ldg(meta + h);
+    double v[kFields];
+    if (m != -1) {
+      const double* p = m >= 0 ? A.qold + (long long)m * NZ + kz
+                               : A.out + (long long)(-2 - m) * kFields * NZ + kz;
+      const long long ld = m >= 0 ? A.old_NG : (long long)NZ;
+#pragma unroll
+      for (int f = 0; f < kFields; ++f) v[f] = __ldg(p + f * ld);
+    } else {
+      const int n1 = A.N + 1, Nq = n1 * n1;
+#pragma unroll
+      for (int f = 0; f < kFields; ++f) v[f] = 0.0;
+      const int end = qt_ptr[h + 1];
+      for (int e = qt_ptr[h]; e < end; ++e) {
+        const int src = qt_src[e], col = src / Nq, ab = src - col * Nq;
+        const int* o = A.org + (long long)col * 6;
+        // w_a w_b hx hy / 4 of the source's column, times the entry's weight
+        const double w = qt_w[e] * (c_tw[A.N][ab % n1] * c_tw[A.N][ab / n1] *
+                                    (A.hxy / (double)(1ll << (2 * A.new_level[col]))));
+        if (o[0] != 0) {
+          const double* p = A.out + (long long)src * kFields * NZ + kz;
+#pragma unroll
+          for (int f = 0; f < kFields; ++f) v[f] = fma(w, __ldg(p + f * (long long)NZ), v[f]);
+          continue;
+        }
+        const int hm = A.old_hmap[(long long)o[1] * Nq + ab];
+        if (hm >= 0) {
+          const double* p = A.qold + (long long)hm * NZ + kz;
+#pragma unroll
+          for (int f = 0; f < kFields; ++f) v[f] = fma(w, __ldg(p + f * A.old_NG), v[f]);
+        } else {
+          const int k = -1 - hm;
+          double u[kFields] = {0, 0, 0, 0, 0};
+          for (int i = 0; i < n1; ++i) {
+            const double wi = A.old_hang_w[k * n1 + i];
+            const double* p = A.qold + (long long)A.old_hang_h[k * n1 + i] * NZ + kz;
+#pragma unroll
+            for (int f = 0; f < kFields; ++f) u[f] += wi * __ldg(p + f * A.old_NG);
           }
-      } else {
-        for (int s = 0; s < 4; ++s) {
-          const int ca = s & 1, cb = s >> 1;
-          for (int m = 0; m < n1; ++m)
-            for (int n = 0; n < n1; ++n) {
-              const double w = 0.25 * c_R[N][ca][i * n1 + m] * c_R[N][cb][j * n1 + n];
-              for (int f = 0; f < kFields; ++f) r[f] += w * sQ[s][f][m + n1 * n + Nq * c];
-            }
+#pragma unroll
+          for (int f = 0; f < kFields; ++f) v[f] = fma(w, u[f], v[f]);
         }
       }
-      const double wJ = wJ1 * A.hzk[k];
-      for (int f = 0; f < kFields; ++f) r[f] *= wJ;
-      if (c == 0 && k > 0)
-        for (int f = 0; f < kFields; ++f) r[f] += sC[(k - 1) & 1][f][ab];
-      if (c == N && k < A.nz - 1) {
-        for (int f = 0; f < kFields; ++f) sC[k & 1][f][ab] = r[f];
-      } else {
-        double* dst = A.out + ((long long)((long long)col * Nq + ab) * kFields) * A.NZ + kz;
-        for (int f = 0; f < kFields; ++f) dst[(long long)f * A.NZ] = r[f];
+      // coupled nodes keep b as the right-hand side of their block solve
+      if (!coupled[h]) {
+#pragma unroll
+        for (int f = 0; f < kFields; ++f) v[f] *= Minv_h[h];
+      }
+    }
+#pragma unroll
+    for (int f = 0; f < kFields; ++f) q[(size_t)f * NG + g] = v[f];
+  }
+}
+
+// Sums over the block of NR values per thread, the same in every thread.
+template <typename T, int NR>
+__device__ __forceinline__ void block_sums(T (&v)[NR], T* red) {
+#pragma unroll
+  for (int i = 0; i < NR; ++i)
+    for (int o = 16; o > 0; o >>= 1) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0)
+#pragma unroll
+    for (int i = 0; i < NR; ++i) red[(threadIdx.x >> 5) * NR + i] = v[i];
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < NR; ++i) {
+    T s = (T)0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w * NR + i];
+    v[i] = s;
+  }
+}
+
+// Coupled blocks, A x = b for NR right-hand sides (field, level) of one block
+// at a time.  As a float64 conjugate gradient, one CTA per right-hand side,
+// this was bound by the float64 pipe (84 % busy, 489 us on 113 k elements with
+// 4 blocks of about 780 nodes and 165 right-hand sides; 396 us now, bound by the
+// latency of the inner iteration).  Now the float64 work
+// is the residual alone: with the symmetrically scaled matrix S A S (S =
+// diag(A)^-1/2, entries of order 1, float32) a float32 conjugate gradient finds
+// the correction to 1e-5, x and r = b - A x are updated in float64, and the
+// residual falls by that factor per pass until it is at rounding level
+// (1e-15 of the right-hand side; a pass that no longer helps ends it too, if
+// the residual is below 3e-14).  The matrix is read once for NR right-hand sides.
+constexpr int kCgThreads = 512, kCgOuter = 12, kCgInner = 200;
+template <int NR>
+__global__ void __launch_bounds__(kCgThreads)
+transfer_cg(const int* __restrict__ comp_ptr, const int* __restrict__ nodes, const int* __restrict__ A_ptr,
+            const int* __restrict__ A_col, const double* __restrict__ A_val, const float* __restrict__ A32,
+            const double* __restrict__ S, long long NG, int NZ, double* q, int* status) {
+  extern __shared__ double sm[];
+  __shared__ double red64[kCgThreads / 32 * NR];
+  float* red = reinterpret_cast<float*>(red64);
+  const int beg = comp_ptr[blockIdx.x], n = comp_ptr[blockIdx.x + 1] - beg;
+  const int rhs0 = blockIdx.y * NR, nrhs = kFields * NZ;
+  double* x = sm;                                  // [n][NR]
+  double* r = x + (size_t)n * NR;
+  float* p = reinterpret_cast<float*>(r + (size_t)n * NR);
+  float* Ap = p + (size_t)n * NR;
+  double* d = reinterpret_cast<double*>(p);        // the correction, over p and Ap
+  float* z = Ap + (size_t)n * NR;                  // scaled residual of the inner iteration
+  float* y = z + (size_t)n * NR;                   // its solution
+  const int t = threadIdx.x, nt = blockDim.x;
+  auto at = [&](int a, int i) {
+    const int rhs = rhs0 + i, f = rhs / NZ, kz = rhs - f * NZ;
+    return (long long)f * NG + (long long)nodes[beg + a] * NZ + kz;
+  };
+  // r -= A v
+  auto residual = [&](const double* v) {
+    for (int a = t; a < n; a += nt) {
+      double s[NR];
+#pragma unroll
+      for (int i = 0; i < NR; ++i) s[i] = r[a * NR + i];
+      for (int e = A_ptr[beg + a]; e < A_ptr[beg + a + 1]; ++e) {
+        const double w = -A_val[e];
+        const int c = A_col[e];
+#pragma unroll
+        for (int i = 0; i < NR; ++i) s[i] = fma(w, v[c * NR + i], s[i]);
+      }
+#pragma unroll
+      for (int i = 0; i < NR; ++i) r[a * NR + i] = s[i];
+    }
+  };
+  auto norms = [&](double (&v)[NR]) {
+#pragma unroll
+    for (int i = 0; i < NR; ++i) v[i] = 0.0;
+    for (int a = t; a < n; a += nt) {
+      const double s = S[beg + a];
+#pragma unroll
+      for (int i = 0; i < NR; ++i) {
+        const double u = r[a * NR + i] * s;
+        v[i] = fma(u, u, v[i]);
+      }
+    }
+    block_sums<double, NR>(v, red64);
+  };
+  for (int a = t; a < n; a += nt) {
+    const double s = S[beg + a];
+#pragma unroll
+    for (int i = 0; i < NR; ++i) {
+      const double b = rhs0 + i < nrhs ? q[at(a, i)] : 0.0;
+      r[a * NR + i] = b;
+      x[a * NR + i] = b * s * s;
+    }
+  }
+  __syncthreads();
+  double bb[NR], rr[NR], last[NR];
+  norms(bb);
+  residual(x);
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < NR; ++i) last[i] = 1e300;
+  bool done = false;
+  for (int outer = 0; outer <= kCgOuter; ++outer) {
+    norms(rr);
+    done = true;
+    double up[NR], dn[NR];   // scale of the inner right-hand side, and back
+#pragma unroll
+    for (int i = 0; i < NR; ++i) {
+      const bool ok = rr[i] <= 1e-30 * bb[i] || (rr[i] >= 0.25 * last[i] && rr[i] <= 1e-27 * bb[i]);
+      done = done && ok;
+      last[i] = rr[i];
+      dn[i] = ok ? 0.0 : sqrt(rr[i]);
+      up[i] = ok ? 0.0 : 1.0 / dn[i];
+    }
+    if (done || outer == kCgOuter) break;
+    float rz[NR];
+#pragma unroll
+    for (int i = 0; i < NR; ++i) rz[i] = 0.f;
+    for (int a = t; a < n; a += nt) {
+      const double s = S[beg + a];
+#pragma unroll
+      for (int i = 0; i < NR; ++i) {
+        const float u = (float)(r[a * NR + i] * s * up[i]);
+        z[a * NR + i] = p[a * NR + i] = u;
+        y[a * NR + i] = 0.f;
+        rz[i] = fmaf(u, u, rz[i]);
+      }
+    }
+    block_sums<float, NR>(rz, red);
+    for (int it = 0; it < kCgInner; ++it) {
+      float pap[NR];
+#pragma unroll
+      for (int i = 0; i < NR; ++i) pap[i] = 0.f;
+      for (int a = t; a < n; a += nt) {
+        float s[NR];
+#pragma unroll
+        for (int i = 0; i < NR; ++i) s[i] = 0.f;
+        for (int e = A_ptr[beg + a]; e < A_ptr[beg + a + 1]; ++e) {
+          const float w = A32[e];
+          const int c = A_col[e];
+#pragma unroll
+          for (int i = 0; i < NR; ++i) s[i] = fmaf(w, p[c * NR + i], s[i]);
+        }
+#pragma unroll
+        for (int i = 0; i < NR; ++i) {
+          Ap[a * NR + i] = s[i];
+          pap[i] = fmaf(p[a * NR + i], s[i], pap[i]);
+        }
+      }
+      block_sums<float, NR>(pap, red);
+      float rz2[NR], alpha[NR];
+#pragma unroll
+      for (int i = 0; i < NR; ++i) {
+        alpha[i] = pap[i] > 0.f ? rz[i] / pap[i] : 0.f;
+        rz2[i] = 0.f;
+      }
+      for (int a = t; a < n; a += nt) {
+#pragma unroll
+        for (int i = 0; i < NR; ++i) {
+          y[a * NR + i] = fmaf(alpha[i], p[a * NR + i], y[a * NR + i]);
+          const float u = fmaf(-alpha[i], Ap[a * NR + i], z[a * NR + i]);
+          z[a * NR + i] = u;
+          rz2[i] = fmaf(u, u, rz2[i]);
+        }
+      }
+      block_sums<float, NR>(rz2, red);
+      float worst = 0.f;
+#pragma unroll
+      for (int i = 0; i < NR; ++i) worst = fmaxf(worst, rz2[i]);
+      if (!(worst > 1e-10f)) break;   // the inner right-hand side has norm 1 (or 0)
+      for (int a = t; a < n; a += nt) {
+#pragma unroll
+        for (int i = 0; i < NR; ++i) {
+          const float beta = rz[i] > 0.f ? rz2[i] / rz[i] : 0.f;
+          p[a * NR + i] = fmaf(beta, p[a * NR + i], z[a * NR + i]);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < NR; ++i) rz[i] = rz2[i];
+      __syncthreads();
+    }
+    __syncthreads();
+    for (int a = t; a < n; a += nt) {
+      const double s = S[beg + a];
+#pragma unroll
+      for (int i = 0; i < NR; ++i) {
+        const double u = (double)y[a * NR + i] * (s * dn[i]);
+        d[a * NR + i] = u;
+        x[a * NR + i] += u;
       }
     }
     __syncthreads();
-  }
-}
-
-__global__ void __launch_bounds__(256)
-transfer_gather(const double* sc, const int* qt_ptr, const int* qt_src, const double* qt_w,
-                const double* Minv_h, const double* Minv_z, const int* coupled, long long NG,
-                int NZ, double* q) {
-  for (long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x; g < NG;
-       g += (long long)gridDim.x * blockDim.x) {
-    const long long h = g / NZ;
-    const int kz = (int)(g - h * NZ);
-    const int beg = qt_ptr[h], end = qt_ptr[h + 1];
-    double acc[kFields] = {0, 0, 0, 0, 0};
-    for (int e = beg; e < end; ++e) {
-      const double w = qt_w[e];
-      const double* p = sc + (long long)qt_src[e] * kFields * NZ + kz;
-      for (int f = 0; f < kFields; ++f) acc[f] += w * p[(long long)f * NZ];
-    }
-    // coupled nodes keep b / M_z(kz) as the right-hand side of their block solve
-    const double s = coupled[h] ? Minv_z[kz] : Minv_h[h] * Minv_z[kz];
-    for (int f = 0; f < kFields; ++f) q[(long long)f * NG + g] = acc[f] * s;
-  }
-}
-
-__device__ double block_sum(double v, double* red) {
-  const int t = threadIdx.x;
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  __syncthreads();
-  if ((t & 31) == 0) red[t >> 5] = v;
-  __syncthreads();
-  double s = 0.0;
-  const int nw = (blockDim.x + 31) >> 5;
-  for (int w = 0; w < nw; ++w) s += red[w];
-  return s;
-}
-
-// one CTA per (component, field, level); dynamic smem 5 n doubles
-__global__ void __launch_bounds__(256)
-transfer_cg(const int* comp_ptr, const int* nodes, const int* A_ptr, const int* A_col,
-            const double* A_val, long long NG, int NZ, double* q, int max_iter, int* status) {
-  extern __shared__ double sm[];
-  __shared__ double red[32];
-  const int comp = blockIdx.x;
-  const int f = blockIdx.y / NZ, kz = blockIdx.y % NZ;
-  const int beg = comp_ptr[comp], n = comp_ptr[comp + 1] - beg;
-  double* x = sm;
-  double* r = sm + n;
-  double* p = sm + 2 * n;
-  double* Ap = sm + 3 * n;
-  double* dinv = sm + 4 * n;
-  const int t = threadIdx.x;
-  double bb = 0.0;
-  for (int a = t; a < n; a += blockDim.x) {
-    const int row = beg + a;
-    double d = 0.0;
-    for (int e = A_ptr[row]; e < A_ptr[row + 1]; ++e)
-      if (A_col[e] == a) d = A_val[e];
-    dinv[a] = 1.0 / d;
-    const double b = q[(long long)f * NG + (long long)nodes[row] * NZ + kz];
-    r[a] = b;            // rhs stored in r until x0 is formed
-    bb += b * b;
-  }
-  bb = block_sum(bb, red);
-  for (int a = t; a < n; a += blockDim.x) x[a] = r[a] * dinv[a];
-  __syncthreads();
-  // r = b - A x0
-  for (int a = t; a < n; a += blockDim.x) {
-    const int row = beg + a;
-    double s = 0.0;
-    for (int e = A_ptr[row]; e < A_ptr[row + 1]; ++e) s += A_val[e] * x[A_col[e]];
-    Ap[a] = r[a] - s;
-  }
-  __syncthreads();
-  double rz = 0.0;
-  for (int a = t; a < n; a += blockDim.x) {
-    r[a] = Ap[a];
-    p[a] = r[a] * dinv[a];
-    rz += r[a] * p[a];
-  }
-  rz = block_sum(rz, red);
-  const double tol2 = 1e-30 * bb;
-  int it = 0;
-  for (; it < max_iter; ++it) {
-    double rr = 0.0;
-    for (int a = t; a < n; a += blockDim.x) rr += r[a] * r[a];
-    rr = block_sum(rr, red);
-    if (rr <= tol2) break;
-    double pAp = 0.0;
-    for (int a = t; a < n; a += blockDim.x) {
-      const int row = beg + a;
-      double s = 0.0;
-      for (int e = A_ptr[row]; e < A_ptr[row + 1]; ++e) s += A_val[e] * p[A_col[e]];
-      Ap[a] = s;
-      pAp += p[a] * s;
-    }
-    pAp = block_sum(pAp, red);
-    const double alpha = rz / pAp;
-    double rz2 = 0.0;
-    for (int a = t; a < n; a += blockDim.x) {
-      x[a] += alpha * p[a];
-      r[a] -= alpha * Ap[a];
-      rz2 += r[a] * r[a] * dinv[a];
-    }
-    rz2 = block_sum(rz2, red);
-    const double beta = rz2 / rz;
-    rz = rz2;
-    for (int a = t; a < n; a += blockDim.x) p[a] = r[a] * dinv[a] + beta * p[a];
+    residual(d);
     __syncthreads();
   }
-  if (it == max_iter && t == 0) atomicOr(status, 2);
-  for (int a = t; a < n; a += blockDim.x)
-    q[(long long)f * NG + (long long)nodes[beg + a] * NZ + kz] = x[a];
+  if (!done && t == 0) atomicOr(status, 2);
+  for (int a = t; a < n; a += nt) {
+#pragma unroll
+    for (int i = 0; i < NR; ++i)
+      if (rhs0 + i < nrhs) q[at(a, i)] = x[a * NR + i];
+  }
 }
 
 // Build the coupled blocks of A_h = Q_h^T W_h Q_h on the host (once per mesh).
@@ -385,6 +573,15 @@ static int build_coupled_blocks(Mesh& m) {
     }
     A_ptr.push_back((int)A_col.size());
   }
+  // S = diag(A)^-1/2 and S A S in float32
+  std::vector<double> sd(rows.size());
+  for (size_t a = 0; a < rows.size(); ++a)
+    for (auto& e : rows[a])
+      if (comp_ptr[cid[nodes[a]]] + e.first == (int)a) sd[a] = 1.0 / std::sqrt(e.second);
+  std::vector<float> A32(A_val.size());
+  for (size_t a = 0; a < rows.size(); ++a)
+    for (int e = A_ptr[a]; e < A_ptr[a + 1]; ++e)
+      A32[e] = (float)(A_val[e] * sd[a] * sd[comp_ptr[cid[nodes[a]]] + A_col[e]]);
   std::vector<int> cpl(nh);
   for (long long h = 0; h < nh; ++h) cpl[h] = coupled[h];
   D.n_comp = (int)comps.size();
@@ -397,17 +594,34 @@ static int build_coupled_blocks(Mesh& m) {
     if (!v.empty()) SEM_CUDA_TRY(cudaMemcpy(dst, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice));
     return SEM_OK;
   };
+  // tr_coupled last: it marks the tables as complete
   int rc;
+  const std::vector<int> meta(nh, -1);
   if ((rc = up(D.tr_comp_ptr, comp_ptr)) || (rc = up(D.tr_nodes, nodes)) || (rc = up(D.tr_A_ptr, A_ptr)) ||
-      (rc = up(D.tr_A_col, A_col)) || (rc = up(D.tr_A_val, A_val)) || (rc = up(D.tr_coupled, cpl)))
+      (rc = up(D.tr_A_col, A_col)) || (rc = up(D.tr_A_val, A_val)) || (rc = up(D.tr_A32, A32)) ||
+      (rc = up(D.tr_S, sd)) || (rc = up(D.tr_meta, meta)) || (rc = up(D.tr_coupled, cpl)))
     return rc;
   return SEM_OK;
 }
 
 template <int N>
 static void launch_local(const TrArgs& A, int ncol, cudaStream_t st) {
-  constexpr int P = (N + 1) * (N + 1) * (N + 1);
-  transfer_local<N><<<ncol, (P + 31) / 32 * 32, 0, st>>>(A);
+  // as few passes of at most kTrThreads threads over a column's (field, level)
+  // pairs as fit, of equal size
+  const int items = kFields * A.NZ, passes = (items + kTrThreads - 1) / kTrThreads;
+  const int nt = ((items + passes - 1) / passes + 31) / 32 * 32;
+  transfer_local<N><<<ncol, nt, 0, st>>>(A);
+}
+
+template <int NR>
+static int launch_cg(Mesh& m, double* q, cudaStream_t st) {
+  DeviceTables& D = *m.dev;
+  const size_t smem = (size_t)32 * NR * D.max_comp;
+  SEM_CUDA_TRY(cudaFuncSetAttribute(transfer_cg<NR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const dim3 grid(D.n_comp, (kFields * m.NZ + NR - 1) / NR);
+  transfer_cg<NR><<<grid, kCgThreads, smem, st>>>(D.tr_comp_ptr, D.tr_nodes, D.tr_A_ptr, D.tr_A_col, D.tr_A_val,
+                                                  D.tr_A32, D.tr_S, m.NG, m.NZ, q, D.status);
+  return SEM_OK;
 }
 
 int launch_transfer(Mesh& o, Mesh& m, const double* qold, double* qnew, cudaStream_t st) {
@@ -416,6 +630,7 @@ int launch_transfer(Mesh& o, Mesh& m, const double* qold, double* qnew, cudaStre
   if ((rc = build_coupled_blocks(m))) return rc;
   DeviceTables& D = *m.dev;
   DeviceTables& Do = *o.dev;
+  if (m.NG >= (1ll << 31)) return fail(SEM_ERR_ARG, "mesh too large for 32-bit node indexing");
   if (o.NZ != m.NZ || o.N != m.N) return fail(SEM_ERR_ARG, "meshes differ in N or layering");
   TrArgs A;
   A.qold = qold;
@@ -426,14 +641,9 @@ int launch_transfer(Mesh& o, Mesh& m, const double* qold, double* qnew, cudaStre
   A.org = D.org;
   A.new_level = D.col_level;
   A.out = (double*)D.scratch;
-  A.nz = m.nz;
+  A.N = m.N;
   A.NZ = m.NZ;
-  A.Lx = m.Lx;
-  A.Ly = m.Ly;
-  A.Lz = m.Lz;
-  A.nx = m.nx;
-  A.ny = m.ny;
-  A.hzk = D.hzk;
+  A.hxy = m.hx(0) * m.hy(0) * 0.25;
   const int nc = (int)m.Ncol();
   switch (m.N) {
     case 2: launch_local<2>(A, nc, st); break;
@@ -444,17 +654,21 @@ int launch_transfer(Mesh& o, Mesh& m, const double* qold, double* qnew, cudaStre
     default: return fail(SEM_ERR_UNSUPPORTED, "order N not compiled");
   }
   SEM_CUDA_TRY(cudaGetLastError());
-  long long blocks = std::min<long long>((m.NG + 255) / 256, 152 * 8);
-  transfer_gather<<<(int)blocks, 256, 0, st>>>((const double*)D.scratch, D.qt_ptr, D.qt_src, D.qt_w,
-                                              D.Minv_h, D.Minv_z, D.tr_coupled, m.NG, m.NZ, qnew);
+  transfer_meta<<<(unsigned)((m.NH + 255) / 256), 256, 0, st>>>(
+      A, reinterpret_cast<const int4*>(D.qt_rec_unit), D.tr_coupled, (int)m.NH, D.tr_meta);
+  long long blocks = std::min<long long>((m.NG + 255) / 256, 152 * 64);
+  transfer_gather<<<(int)blocks, 256, 0, st>>>(A, D.tr_meta, D.qt_ptr, D.qt_src, D.qt_w, D.Minv_h, D.tr_coupled,
+                                              (unsigned)m.NG, qnew);
   SEM_CUDA_TRY(cudaGetLastError());
   if (D.n_comp > 0) {
-    const size_t smem = (size_t)5 * D.max_comp * sizeof(double);
-    if (smem > 200 * 1024) return fail(SEM_ERR_UNSUPPORTED, "coupled 2:1 block too large for one CTA");
-    SEM_CUDA_TRY(cudaFuncSetAttribute(transfer_cg, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    dim3 grid(D.n_comp, kFields * m.NZ);
-    transfer_cg<<<grid, 256, smem, st>>>(D.tr_comp_ptr, D.tr_nodes, D.tr_A_ptr, D.tr_A_col, D.tr_A_val,
-                                         m.NG, m.NZ, qnew, 500, D.status);
+    // four right-hand sides per CTA where their vectors fit its shared memory
+    // and the blocks still give every SM one
+    if ((size_t)40 * D.max_comp > 200 * 1024) return fail(SEM_ERR_UNSUPPORTED, "coupled 2:1 block too large for one CTA");
+    int dev = 0, nsm = 152;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    const bool four = (size_t)128 * D.max_comp <= 200 * 1024 && (long long)D.n_comp * kFields * m.NZ >= 4LL * nsm;
+    if ((rc = four ? launch_cg<4>(m, qnew, st) : launch_cg<1>(m, qnew, st))) return rc;
     SEM_CUDA_TRY(cudaGetLastError());
   }
   return SEM_OK;

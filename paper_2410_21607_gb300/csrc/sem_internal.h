@@ -190,6 +190,9 @@ struct DeviceTables {
   int* tr_A_col = nullptr;      // component-local column
   double* tr_A_val = nullptr;
   int* tr_coupled = nullptr;    // [NH] 1 when the node is solved for
+  float* tr_A32 = nullptr;      // S A_h S in float32, S = diag(A_h)^-1/2
+  double* tr_S = nullptr;       // [nodes] S
+  int* tr_meta = nullptr;       // [NH] where each new line comes from (transfer_meta)
   // the params the ref tables were built with
   double ref_key[8] = {0};
   bool ref_valid = false;
