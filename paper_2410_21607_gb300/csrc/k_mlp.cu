@@ -1,6 +1,6 @@
 // Learned refinement flags: per-element features, a 3-layer MLP (136-128-128-3)
-// with bfloat16 tensor-core forward products and float32 accumulation, its
-// backward pass and Adam.
+// with bfloat16 tensor-core products and float32 accumulation, its backward
+// pass (float32 values as sums of bfloat16 parts) and Adam.
 //
 // The paper's velocity criterion (Sec. 3.1) fires only once intensification
 // has started (Sec. 5); the network predicts the criterion's flags some steps
@@ -73,15 +73,15 @@ __global__ void mlp_refresh(const float* __restrict__ P, __nv_bfloat16* __restri
 }
 
 // Forward pass.  One warp per 16 rows, 4 warps per CTA.  Writes the class
-// probabilities, and in training mode the rounded inputs and activations.
+// probabilities, and in training mode the rounded activations.
 constexpr int FWD_ROWS = 64;
 constexpr size_t FWD_SMEM = (size_t)(W1T_SZ + W2T_SZ + W3T_SZ) * 2 + (2 * HID + 8) * 4;
 
 __global__ void __launch_bounds__(128)
 mlp_forward(const float* __restrict__ X, int n, const __nv_bfloat16* __restrict__ w1t,
             const __nv_bfloat16* __restrict__ w2t, const __nv_bfloat16* __restrict__ w3t,
-            const float* __restrict__ P, float* __restrict__ prob, float* __restrict__ Xr,
-            float* __restrict__ H1r, float* __restrict__ H2r, int8_t* __restrict__ flags) {
+            const float* __restrict__ P, float* __restrict__ prob, __nv_bfloat16* __restrict__ H1r,
+            __nv_bfloat16* __restrict__ H2r, int8_t* __restrict__ flags) {
   extern __shared__ __align__(16) unsigned char sm[];
   __nv_bfloat16* s1 = reinterpret_cast<__nv_bfloat16*>(sm);
   __nv_bfloat16* s2 = s1 + W1T_SZ;
@@ -114,10 +114,6 @@ mlp_forward(const float* __restrict__ X, int n, const __nv_bfloat16* __restrict_
       if (rb < n && c < IN) { y0 = X[(long long)rb * IN + c]; y1 = X[(long long)rb * IN + c + 1]; }
       a[s][2 * h + 0] = pack_bf16(x0, x1);
       a[s][2 * h + 1] = pack_bf16(y0, y1);
-      if (Xr && c < IN) {
-        if (ra < n) { Xr[(long long)ra * IN + c] = bf16r(x0); Xr[(long long)ra * IN + c + 1] = bf16r(x1); }
-        if (rb < n) { Xr[(long long)rb * IN + c] = bf16r(y0); Xr[(long long)rb * IN + c + 1] = bf16r(y1); }
-      }
     }
   }
   // layer 1: 16 column tiles of 8; results become layer 2's A fragments
@@ -138,8 +134,8 @@ mlp_forward(const float* __restrict__ X, int n, const __nv_bfloat16* __restrict_
     h1[t >> 1][(t & 1) * 2 + 0] = pack_bf16(v0, v1);
     h1[t >> 1][(t & 1) * 2 + 1] = pack_bf16(v2, v3);
     if (H1r) {
-      if (ra < n) { H1r[(long long)ra * HID + c] = bf16r(v0); H1r[(long long)ra * HID + c + 1] = bf16r(v1); }
-      if (rb < n) { H1r[(long long)rb * HID + c] = bf16r(v2); H1r[(long long)rb * HID + c + 1] = bf16r(v3); }
+      if (ra < n) *reinterpret_cast<unsigned*>(H1r + (long long)ra * HID + c) = h1[t >> 1][(t & 1) * 2 + 0];
+      if (rb < n) *reinterpret_cast<unsigned*>(H1r + (long long)rb * HID + c) = h1[t >> 1][(t & 1) * 2 + 1];
     }
   }
   // layer 2
@@ -160,8 +156,8 @@ mlp_forward(const float* __restrict__ X, int n, const __nv_bfloat16* __restrict_
     h2[t >> 1][(t & 1) * 2 + 0] = pack_bf16(v0, v1);
     h2[t >> 1][(t & 1) * 2 + 1] = pack_bf16(v2, v3);
     if (H2r) {
-      if (ra < n) { H2r[(long long)ra * HID + c] = bf16r(v0); H2r[(long long)ra * HID + c + 1] = bf16r(v1); }
-      if (rb < n) { H2r[(long long)rb * HID + c] = bf16r(v2); H2r[(long long)rb * HID + c + 1] = bf16r(v3); }
+      if (ra < n) *reinterpret_cast<unsigned*>(H2r + (long long)ra * HID + c) = h2[t >> 1][(t & 1) * 2 + 0];
+      if (rb < n) *reinterpret_cast<unsigned*>(H2r + (long long)rb * HID + c) = h2[t >> 1][(t & 1) * 2 + 1];
     }
   }
   // layer 3: one column tile (3 of 8 used)
@@ -209,9 +205,13 @@ mlp_forward(const float* __restrict__ X, int n, const __nv_bfloat16* __restrict_
 }
 
 // Forward pass on the fifth-generation tensor cores (tcgen05), the
-// default: persistent CTAs of 128 threads (two per SM) keep the weights in
-// shared memory and walk over tiles of 128 rows, thread t owning row t of a
-// tile (tensor memory lane t).  The three layers are GEMMs of M = 128 rows by N = 128 (16
+// default: persistent CTAs of 256 threads (two per SM) keep the weights in
+// shared memory and walk over tiles of 128 rows, threads t and t + 128 owning
+// the halves of row t of a tile (tensor memory lane t).  A thread asks for all
+// of its share of a tile at once, and for the next tile's while this one is
+// computed: the inputs (544 B a row) are what the pass cannot do without, and
+// with 128 threads loading and rounding in turn their latency was most of its
+// time (65536 rows: 54 us, now 28).  The three layers are GEMMs of M = 128 rows by N = 128 (16
 // for the 3 logits) by K = 144 (the 136 inputs padded) or 128, as
 // tcgen05.mma.cta_group::1.kind::f16 with bfloat16 operands from shared memory
 // (K-major, no swizzle: core matrices of 8 rows x 8 bfloat16) and float32
@@ -234,11 +234,24 @@ __device__ __forceinline__ int boff(int r, int k, int kc) {
   return (r & 7) * 16 + (k & 7) * 2 + (k >> 3) * 128 + (r >> 3) * (kc * 128);
 }
 
-__global__ void __launch_bounds__(TC_ROWS, 2)
+constexpr int TC_T = 256, TC_XV = TC_ROWS * (IN / 4) / TC_T;   // threads; float4 of a tile per thread
+static_assert(TC_T == 256 && TC_XV * TC_T == TC_ROWS * (IN / 4), "a tile divides evenly");
+// The j-th float4 (row r, columns k..k+3) of a 128 x 136 tile for this thread
+// of WARPS warps: half a warp takes 8 rows x 32 bytes, whose rounded values fill one
+// core matrix (no bank conflicts; a row's worth of neighbouring lanes would
+// fall on the same banks).
+template <int WARPS>
+__device__ __forceinline__ void input_at(int j, int& r, int& k) {
+  const int lane = threadIdx.x & 31, unit = (j * WARPS + (int)(threadIdx.x >> 5)) * 2 + (lane >> 4);
+  const int g = unit / (IN / 8), c = unit - g * (IN / 8);
+  r = g * 8 + ((lane >> 1) & 7);
+  k = c * 8 + (lane & 1) * 4;
+}
+__global__ void __launch_bounds__(TC_T, 2)
 mlp_forward_tc(const float* __restrict__ X, int n, const __nv_bfloat16* __restrict__ w1t,
                const __nv_bfloat16* __restrict__ w2t, const __nv_bfloat16* __restrict__ w3t,
-               const float* __restrict__ P, float* __restrict__ prob, float* __restrict__ Xr,
-               float* __restrict__ H1r, float* __restrict__ H2r, int8_t* __restrict__ flags, int* err) {
+               const float* __restrict__ P, float* __restrict__ prob, __nv_bfloat16* __restrict__ H1r,
+               __nv_bfloat16* __restrict__ H2r, int8_t* __restrict__ flags, int* err) {
   extern __shared__ __align__(1024) unsigned char sm_tc[];
   unsigned char* sA = sm_tc;
   unsigned char* sW1 = sA + TC_X_BYTES;
@@ -247,24 +260,40 @@ mlp_forward_tc(const float* __restrict__ X, int n, const __nv_bfloat16* __restri
   float* sb = reinterpret_cast<float*>(sW3 + TC_W3_BYTES);   // b1 | b2 | b3 (16)
   uint64_t* mbar = reinterpret_cast<uint64_t*>(sb + 2 * HID + 16);
   uint32_t* taddr_s = reinterpret_cast<uint32_t*>(mbar + 1);
-  const int t = threadIdx.x, warp = t >> 5;
+  const int t = threadIdx.x, warp = t >> 5, rl = t & 127, half = t >> 7;
+  const int ntiles = (n + TC_ROWS - 1) / TC_ROWS;
+  // inputs: float4 loads, 8 rows x 64 contiguous bytes per warp
+  float4 xv[TC_XV];
+  auto load = [&](int tile) {
+    const long long row0 = (long long)tile * TC_ROWS;
+#pragma unroll
+    for (int j = 0; j < TC_XV; ++j) {
+      int r, k;
+      input_at<TC_T / 32>(j, r, k);
+      xv[j] = row0 + r < n ? __ldg(reinterpret_cast<const float4*>(X + (row0 + r) * IN + k))
+                           : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  };
+  load(blockIdx.x);
   // weights: 8 bfloat16 (16 bytes) per core-matrix row; the transposed
   // arrays hold row n of W^T with k contiguous (zero beyond the inputs)
-  for (int i = t; i < HID * 18; i += TC_ROWS) {
+#pragma unroll
+  for (int i = t; i < HID * 18; i += TC_T) {
     const int nn = i / 18, c = i % 18;
     *reinterpret_cast<uint4*>(sW1 + boff(nn, 8 * c, 18)) = *reinterpret_cast<const uint4*>(w1t + nn * K1P + 8 * c);
   }
-  for (int i = t; i < HID * 16; i += TC_ROWS) {
+#pragma unroll
+  for (int i = t; i < HID * 16; i += TC_T) {
     const int nn = i / 16, c = i % 16;
     *reinterpret_cast<uint4*>(sW2 + boff(nn, 8 * c, 16)) = *reinterpret_cast<const uint4*>(w2t + nn * K2P + 8 * c);
   }
-  for (int i = t; i < 16 * 16; i += TC_ROWS) {
+  for (int i = t; i < 16 * 16; i += TC_T) {
     const int nn = i / 16, c = i % 16;
     const uint4 z = make_uint4(0u, 0u, 0u, 0u);
     *reinterpret_cast<uint4*>(sW3 + boff(nn, 8 * c, 16)) =
         nn < 8 ? *reinterpret_cast<const uint4*>(w3t + nn * K2P + 8 * c) : z;
   }
-  for (int i = t; i < HID; i += TC_ROWS) {
+  for (int i = t; i < HID; i += TC_T) {
     sb[i] = P[OFF_B1 + i];
     sb[HID + i] = P[OFF_B2 + i];
   }
@@ -276,30 +305,26 @@ mlp_forward_tc(const float* __restrict__ X, int n, const __nv_bfloat16* __restri
   tcg::fence_after();
   const uint32_t taddr = *taddr_s, bar = tcg::smem_u32(mbar);
   const uint32_t aA = tcg::smem_u32(sA), a1 = tcg::smem_u32(sW1), a2 = tcg::smem_u32(sW2), a3 = tcg::smem_u32(sW3);
-  const uint32_t lane_addr = taddr + ((uint32_t)(32 * warp) << 16);
+  const uint32_t lane_addr = taddr + ((uint32_t)(32 * (warp & 3)) << 16);
   bool ok = true;
   uint32_t phase = 0;   // completions of the barrier so far (three per tile)
-  const int ntiles = (n + TC_ROWS - 1) / TC_ROWS;
   // persistent: the CTA keeps the weights and walks over tiles of 128 rows
   for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
   const long long row0 = (long long)tile * TC_ROWS;
-  // inputs: the 128 x 136 tile is contiguous; coalesced float4 loads, each
-  // inside one row (136 is a multiple of 4), rounded to bfloat16
-  for (int i = t; i < TC_ROWS * (IN / 4); i += TC_ROWS) {
-    const int r = i / (IN / 4), k = 4 * (i % (IN / 4));
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (row0 + r < n) v = *reinterpret_cast<const float4*>(X + (row0 + r) * IN + k);
-    const unsigned lo = pack_bf16(v.x, v.y), hi = pack_bf16(v.z, v.w);
-    *reinterpret_cast<uint2*>(sA + boff(r, k, 18)) = make_uint2(lo, hi);
-    if (Xr && row0 + r < n)
-      *reinterpret_cast<float4*>(Xr + (row0 + r) * IN + k) = make_float4(bf16r(v.x), bf16r(v.y), bf16r(v.z), bf16r(v.w));
+#pragma unroll
+  for (int j = 0; j < TC_XV; ++j) {
+    int r, k;
+    input_at<TC_T / 32>(j, r, k);
+    *reinterpret_cast<uint2*>(sA + boff(r, k, 18)) =
+        make_uint2(pack_bf16(xv[j].x, xv[j].y), pack_bf16(xv[j].z, xv[j].w));
   }
-  *reinterpret_cast<uint4*>(sA + boff(t, IN, 18)) = make_uint4(0u, 0u, 0u, 0u);   // k = 136..143
+  if (half == 0) *reinterpret_cast<uint4*>(sA + boff(rl, IN, 18)) = make_uint4(0u, 0u, 0u, 0u);   // k = 136..143
+  if (tile + (int)gridDim.x < ntiles) load(tile + gridDim.x);
   tcg::fence_async_smem();
   tcg::fence_before();
   __syncthreads();
   tcg::fence_after();
-  const long long row = row0 + t;
+  const long long row = row0 + rl;
   // layer 1: 9 steps of K = 16 (two core matrices each)
   if (t == 0) {
     for (int ks = 0; ks < 9; ++ks)
@@ -311,23 +336,20 @@ mlp_forward_tc(const float* __restrict__ X, int n, const __nv_bfloat16* __restri
   ++phase;
   tcg::fence_after();
   // hidden layers: bias, ReLU, bfloat16, written as the next A operand
-  auto hidden = [&](uint32_t col0, const float* bias, float* Hr) {
+  auto hidden = [&](uint32_t col0, const float* bias, __nv_bfloat16* Hr) {
 #pragma unroll 1
-    for (int c0 = 0; c0 < HID; c0 += 16) {
+    for (int c0 = 64 * half; c0 < 64 * half + 64; c0 += 16) {
       float v[16];
       tcg::ld16(lane_addr + col0 + c0, v);
       tcg::wait_ld();
 #pragma unroll
       for (int q = 0; q < 16; ++q) v[q] = bf16r(fmaxf(v[q] + bias[c0 + q], 0.f));
 #pragma unroll
-      for (int h = 0; h < 2; ++h)
-        *reinterpret_cast<uint4*>(sA + boff(t, c0 + 8 * h, 16)) =
-            make_uint4(pack_bf16(v[8 * h + 0], v[8 * h + 1]), pack_bf16(v[8 * h + 2], v[8 * h + 3]),
-                       pack_bf16(v[8 * h + 4], v[8 * h + 5]), pack_bf16(v[8 * h + 6], v[8 * h + 7]));
-      if (Hr && row < n) {
-#pragma unroll
-        for (int q = 0; q < 16; q += 4)
-          *reinterpret_cast<float4*>(Hr + row * HID + c0 + q) = make_float4(v[q], v[q + 1], v[q + 2], v[q + 3]);
+      for (int h = 0; h < 2; ++h) {
+        const uint4 w = make_uint4(pack_bf16(v[8 * h + 0], v[8 * h + 1]), pack_bf16(v[8 * h + 2], v[8 * h + 3]),
+                                   pack_bf16(v[8 * h + 4], v[8 * h + 5]), pack_bf16(v[8 * h + 6], v[8 * h + 7]));
+        *reinterpret_cast<uint4*>(sA + boff(rl, c0 + 8 * h, 16)) = w;
+        if (Hr && row < n) *reinterpret_cast<uint4*>(Hr + row * HID + c0 + 8 * h) = w;
       }
     }
   };
@@ -359,7 +381,7 @@ mlp_forward_tc(const float* __restrict__ X, int n, const __nv_bfloat16* __restri
   ok = __syncthreads_and(ok && tcg::mbar_wait(bar, phase & 1));
   ++phase;
   tcg::fence_after();
-  if (ok) {
+  if (ok && half == 0) {
     float z[16];
     tcg::ld16(lane_addr, z);
     tcg::wait_ld();
@@ -380,7 +402,7 @@ mlp_forward_tc(const float* __restrict__ X, int n, const __nv_bfloat16* __restri
         flags[row] = (int8_t)(cls - 1);
       }
     }
-  } else if ((t & 31) == 0) {
+  } else if (!ok && (t & 31) == 0) {
     atomicOr(err, 4);
   }
   // the next tile overwrites the A operand and the accumulators: every
@@ -394,8 +416,7 @@ mlp_forward_tc(const float* __restrict__ X, int n, const __nv_bfloat16* __restri
   if (warp == 0) tcg::dealloc(taddr, 256);
 }
 
-// dZ3 = w_y (p - onehot) / sum(w_y); loss partial sums into acc[0] (sum w_y
-// (-log p_y)) -- acc[1] holds sum w_y from mlp_wsum.
+// sum of the rows' class weights into acc[1]
 __global__ void mlp_wsum(const int8_t* __restrict__ y, int n, float w0, float w1, float w2,
                          double* __restrict__ acc) {
   __shared__ double red[256];
@@ -413,90 +434,326 @@ __global__ void mlp_wsum(const int8_t* __restrict__ y, int n, float w0, float w1
   if (threadIdx.x == 0) atomicAdd(acc + 1, red[0]);
 }
 
-__global__ void mlp_dz3(const float* __restrict__ prob, const int8_t* __restrict__ y, int n, float w0,
-                        float w1, float w2, const double* __restrict__ acc_in, float* __restrict__ dz,
-                        double* __restrict__ acc) {
-  __shared__ double red[256];
-  const float inv = (float)(1.0 / acc_in[1]);
-  double l = 0.0;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const int c = y[i];
-    const float w = c == 0 ? w0 : (c == 1 ? w1 : w2);
-    for (int k = 0; k < OUT; ++k) dz[(long long)i * OUT + k] = w * inv * (prob[(long long)i * OUT + k] - (k == c ? 1.f : 0.f));
-    l += (double)w * -log((double)prob[(long long)i * OUT + c]);
+// Backward pass on the tensor cores, one persistent CTA per SM walking over
+// tiles of 128 rows.  Per tile, with dZ3 = w_y (p - onehot) / sum(w_y):
+//   gW3 += H2^T dZ3,  dZ2 = (dZ3 W3^T) [H2 > 0],  gW2 += H1^T dZ2,
+//   dZ1 = (dZ2 W2^T) [H1 > 0],                     gW1 += X^T dZ1.
+// The rounded inputs, activations and weights are bfloat16 values, the dZ are
+// float32: each dZ is split into three bfloat16 parts whose sum is exact (8
+// bits of the significand each), so every product is exact and the sums are
+// float32, as in a float32 matrix product.  The tensor cores truncate when they
+// add to an accumulator (24 steps on a large one left 5e-7, over all of a CTA's
+// tiles 1e-6), so the small parts go first, the large part's eight steps are
+// shared by two accumulators where tensor memory has room, and every tile's
+// sums are added to float32 registers, rounding to nearest: the error against
+// float64 is then that of float32 fused multiply-adds.  The weight gradients
+// are formed as gW^T (rows are the features of dZ, so that X's 136 + 8 columns
+// are the N extent); a column of ones beside X and H1 gives the bias gradients
+// in the same products.  A tile is stored once,
+// in core matrices of 8 rows x 8 features: read along the features it is the
+// K-major operand of the dZ1 product, read along the rows the MN-major operand
+// of the gradient products.  Each CTA writes its sums, mlp_sum adds them in
+// order (deterministic).  65536 rows: 68 us; 32x32 float32 tiles on the CUDA cores
+// took 240 + 224 + 123 + 123 + 91 us for the five products and 180 us for the
+// masks and bias sums between them, each with its own pass over memory.
+constexpr int BW_T = 512;
+constexpr int BW_X = 0, BW_H = BW_X + 128 * 144 * 2, BW_D = BW_H + 128 * 144 * 2, BW_W2 = BW_D + 3 * 128 * HID * 2;
+constexpr int BW_D3 = BW_W2 + HID * HID * 2, BW_W3 = BW_D3 + 128 * 16 * 2, BW_RED = BW_W3 + HID * OUT * 4;
+constexpr int BW_BAR = BW_RED + 16 * 8 * 4;
+constexpr size_t BW_SMEM = BW_BAR + 16;
+// tensor memory columns: dZ1 (two accumulators), gW2, gW3; then gW1 (two)
+constexpr uint32_t BW_C1 = 0, BW_G2 = 256, BW_G3 = 416, BW_G1 = 0;
+constexpr int BW_SUMS = 10;   // groups of 8 gradient columns per thread
+
+// two float32 values as three bfloat16 pairs, x = p[0] + p[1] + p[2] (exact for
+// finite x away from the smallest float32 values): one packed conversion per
+// part, the residuals by the parts' bits
+__device__ __forceinline__ void split3(float a, float b, unsigned (&p)[3]) {
+#pragma unroll
+  for (int s = 0; s < 3; ++s) {
+    p[s] = pack_bf16(a, b);
+    a -= __uint_as_float(p[s] << 16);
+    b -= __uint_as_float(p[s] & 0xffff0000u);
   }
-  red[threadIdx.x] = l;
+}
+// eight values of row r, columns k..k+7, split into the three tiles at D
+__device__ __forceinline__ void put_split(unsigned char* D, int r, int k, const float (&v)[8]) {
+  unsigned q[3][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    unsigned p[3];
+    split3(v[2 * i], v[2 * i + 1], p);
+#pragma unroll
+    for (int s = 0; s < 3; ++s) q[s][i] = p[s];
+  }
+#pragma unroll
+  for (int s = 0; s < 3; ++s)
+    *reinterpret_cast<uint4*>(D + s * 128 * HID * 2 + boff(r, k, 16)) = make_uint4(q[s][0], q[s][1], q[s][2], q[s][3]);
+}
+// v where the bfloat16 activation is positive (neither zero nor NaN), else 0
+__device__ __forceinline__ float masked(unsigned pair, int i, float v) {
+  const unsigned b = (pair >> (16 * (i & 1))) & 0xffffu;
+  return b - 1u < 0x7f80u ? v : 0.f;
+}
+
+__global__ void __launch_bounds__(BW_T, 1)
+mlp_backward_tc(const float* __restrict__ X, const int8_t* __restrict__ y, int n, float w0, float w1, float w2,
+                const float* __restrict__ prob, const __nv_bfloat16* __restrict__ H1,
+                const __nv_bfloat16* __restrict__ H2, const float* __restrict__ R, double* __restrict__ acc,
+                int want_loss, float* __restrict__ part, int* err) {
+  extern __shared__ __align__(1024) unsigned char sm_bw[];
+  unsigned char *sX = sm_bw + BW_X, *sH = sm_bw + BW_H, *sD = sm_bw + BW_D, *sW2 = sm_bw + BW_W2, *sD3 = sm_bw + BW_D3;
+  float* sW3 = reinterpret_cast<float*>(sm_bw + BW_W3);
+  float* sRed = reinterpret_cast<float*>(sm_bw + BW_RED);
+  uint64_t* mbar = reinterpret_cast<uint64_t*>(sm_bw + BW_BAR);
+  uint32_t* slot = reinterpret_cast<uint32_t*>(mbar + 1);
+  const int t = threadIdx.x, warp = t >> 5, r = t & 127, qd = t >> 7;
+  // W2 (input-major rows are K-major for dZ2 W2^T) and W3
+  for (int i = t; i < HID * HID / 8; i += BW_T) {
+    const int a = i / (HID / 8), k = 8 * (i % (HID / 8));
+    const float4* p = reinterpret_cast<const float4*>(R + OFF_W2 + a * HID + k);
+    const float4 u = p[0], v = p[1];
+    *reinterpret_cast<uint4*>(sW2 + boff(a, k, 16)) =
+        make_uint4(pack_bf16(u.x, u.y), pack_bf16(u.z, u.w), pack_bf16(v.x, v.y), pack_bf16(v.z, v.w));
+  }
+  for (int i = t; i < HID * OUT; i += BW_T) sW3[i] = R[OFF_W3 + i];
+  // the columns of ones (136 of X, 128 of H1) and the padding
+  if (qd == 0) {
+    const uint4 one = make_uint4(0x00003f80u, 0u, 0u, 0u), z = make_uint4(0u, 0u, 0u, 0u);
+    *reinterpret_cast<uint4*>(sX + boff(r, IN, 18)) = one;
+    *reinterpret_cast<uint4*>(sH + boff(r, HID, 18)) = one;
+    *reinterpret_cast<uint4*>(sH + boff(r, HID + 8, 18)) = z;
+    *reinterpret_cast<uint4*>(sD3 + boff(r, 8, 2)) = z;
+  }
+  if (warp == 0) tcg::alloc(slot, 512);
+  if (t == 0) tcg::mbar_init(tcg::smem_u32(mbar), 1);
+  tcg::fence_before();
   __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+  tcg::fence_after();
+  const uint32_t taddr = *slot, bar = tcg::smem_u32(mbar);
+  const uint32_t lane = taddr + ((uint32_t)(32 * (warp & 3)) << 16);
+  const uint32_t aX = tcg::smem_u32(sX), aH = tcg::smem_u32(sH), aD = tcg::smem_u32(sD), aW2 = tcg::smem_u32(sW2),
+                 aD3 = tcg::smem_u32(sD3);
+  constexpr uint32_t kTA = 1u << 15, kTB = 1u << 16;   // A, B MN-major
+  constexpr uint32_t TILE = 128 * HID * 2;
+  const bool aligned = ((uintptr_t)X & 15) == 0;   // the mma.sync forward takes any X
+  const float inv = (float)(1.0 / acc[1]);
+  float gb3[3] = {0.f, 0.f, 0.f};
+  // running sums of this thread's gradient columns: group g = qd + 4 i of 8
+  // columns is gW1^T's g-th (g < 18), gW2^T's (g < 36) or gW3's (g < 38)
+  float sum[BW_SUMS][8];
+#pragma unroll
+  for (int i = 0; i < BW_SUMS; ++i)
+#pragma unroll
+    for (int j = 0; j < 8; ++j) sum[i][j] = 0.f;
+  auto add_cols = [&](uint32_t col, int second, float (&v)[8]) {   // v += columns col.. (and col + second..)
+    float a[8], b[8];
+    tcg::ld8(lane + col, a);
+    if (second) tcg::ld8(lane + col + second, b);
+    tcg::wait_ld();
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[j] += second ? a[j] + b[j] : a[j];
+  };
+  double loss = 0.0;
+  bool ok = true;
+  uint32_t phase = 0;
+  // all threads' shared-memory writes before the tensor cores read them
+  auto publish = [&] {
+    tcg::fence_async_smem();
+    tcg::fence_before();
     __syncthreads();
+    tcg::fence_after();
+  };
+  auto wait = [&] {
+    ok = __syncthreads_and(tcg::mbar_wait(bar, phase & 1));
+    ++phase;
+    tcg::fence_after();
+  };
+  const int ntiles = (n + 127) / 128;
+  for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
+    const long long row0 = (long long)tile * 128;
+    const bool in = row0 + r < n;
+#pragma unroll
+    for (int j = 0; j < (TC_XV + 1) / 2; ++j) {
+      int rr, k;
+      input_at<BW_T / 32>(j, rr, k);
+      if (rr >= 128) break;
+      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (row0 + rr < n) {
+        const float* p = X + (row0 + rr) * IN + k;
+        v = aligned ? *reinterpret_cast<const float4*>(p) : make_float4(p[0], p[1], p[2], p[3]);
+      }
+      *reinterpret_cast<uint2*>(sX + boff(rr, k, 18)) = make_uint2(pack_bf16(v.x, v.y), pack_bf16(v.z, v.w));
+    }
+#pragma unroll
+    for (int j = 0; j < 128 * (HID / 8) / BW_T; ++j) {
+      // a warp: 8 rows x 64 bytes
+      const int u = j * (BW_T / 32) + warp, rr = (u >> 2) * 8 + (t & 7), k = 8 * ((u & 3) * 4 + ((t >> 3) & 3));
+      uint4 a = make_uint4(0u, 0u, 0u, 0u), b = a;
+      if (row0 + rr < n) {
+        a = *reinterpret_cast<const uint4*>(H1 + (row0 + rr) * HID + k);
+        b = *reinterpret_cast<const uint4*>(H2 + (row0 + rr) * HID + k);
+      }
+      *reinterpret_cast<uint4*>(sH + boff(rr, k, 18)) = a;
+      *reinterpret_cast<uint4*>(sD + 2 * TILE + boff(rr, k, 16)) = b;   // H2, until dZ2 takes its place
+    }
+    float d3[3] = {0.f, 0.f, 0.f};
+    if (in) {
+      const int c = y[row0 + r];
+      const float w = c == 0 ? w0 : (c == 1 ? w1 : w2);
+#pragma unroll
+      for (int k = 0; k < OUT; ++k) d3[k] = w * inv * (prob[(row0 + r) * OUT + k] - (k == c ? 1.f : 0.f));
+      if (qd == 0 && want_loss) loss += (double)w * -log((double)prob[(row0 + r) * OUT + c]);
+    }
+    if (qd == 0) {
+      // the three parts of dZ3 side by side: columns c + 3 s
+      unsigned p[3], z[3];
+      split3(d3[0], d3[1], p);
+      split3(d3[2], 0.f, z);
+      const unsigned w[5] = {p[0], (z[0] & 0xffffu) | (p[1] << 16), (p[1] >> 16) | (z[1] << 16), p[2], z[2] & 0xffffu};
+      *reinterpret_cast<uint4*>(sD3 + boff(r, 0, 2)) = make_uint4(w[0], w[1], w[2], w[3]);
+      *reinterpret_cast<uint4*>(sD3 + boff(r, 8, 2)) = make_uint4(w[4], 0u, 0u, 0u);
+#pragma unroll
+      for (int k = 0; k < OUT; ++k) gb3[k] += d3[k];
+    }
+    publish();
+    if (t == 0) {
+      // gW3 (M = features of H2, N = 16, K = rows)
+      for (int ks = 0; ks < 8; ++ks)
+        tcg::mma_f16(taddr + BW_G3, tcg::sdesc(aD + 2 * TILE + ks * 4096, 2048, 128),
+                     tcg::sdesc(aD3 + ks * 512, 256, 128), tcg::idesc_bf16(128, 16) | kTA | kTB, ks > 0);
+      tcg::commit(bar);
+    }
+    wait();
+    if (!ok) break;
+    // dZ2, its third part over H2
+#pragma unroll 1
+    for (int k = 32 * qd; k < 32 * qd + 32; k += 8) {
+      const uint4 h = *reinterpret_cast<const uint4*>(sD + 2 * TILE + boff(r, k, 16));
+      const unsigned hw[4] = {h.x, h.y, h.z, h.w};
+      float v[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const float* w = sW3 + (k + i) * OUT;
+        v[i] = masked(hw[i >> 1], i, fmaf(d3[2], w[2], fmaf(d3[1], w[1], d3[0] * w[0])));
+      }
+      put_split(sD, r, k, v);
+    }
+    publish();
+    if (t == 0) {
+      for (int s = 2; s >= 0; --s)
+        for (int ks = 0; ks < 8; ++ks) {   // dZ1 (M = rows, N = features of H1, K = features of dZ2)
+          const int b = s == 0 && ks >= 4;
+          tcg::mma_f16(taddr + BW_C1 + 128 * b, tcg::sdesc(aD + s * TILE + ks * 256, 128, 2048),
+                       tcg::sdesc(aW2 + ks * 256, 128, 2048), tcg::idesc_bf16(128, 128), b ? ks > 4 : (s < 2 || ks > 0));
+        }
+      for (int s = 2; s >= 0; --s)
+        for (int ks = 0; ks < 8; ++ks)   // gW2^T (M = features of dZ2, N = features of H1 and the ones, K = rows)
+          tcg::mma_f16(taddr + BW_G2, tcg::sdesc(aD + s * TILE + ks * 4096, 2048, 128),
+                       tcg::sdesc(aH + ks * 4608, 2304, 128), tcg::idesc_bf16(128, 144) | kTA | kTB, s < 2 || ks > 0);
+      tcg::commit(bar);
+    }
+    wait();
+    if (!ok) break;
+    // dZ1 over dZ2
+#pragma unroll 1
+    for (int k = 32 * qd; k < 32 * qd + 32; k += 8) {
+      float z[8], z2[8], v[8];
+      tcg::ld8(lane + BW_C1 + k, z);
+      tcg::ld8(lane + BW_C1 + 128 + k, z2);
+      tcg::wait_ld();
+      const uint4 h = *reinterpret_cast<const uint4*>(sH + boff(r, k, 18));
+      const unsigned hw[4] = {h.x, h.y, h.z, h.w};
+#pragma unroll
+      for (int i = 0; i < 8; ++i) v[i] = masked(hw[i >> 1], i, z[i] + z2[i]);
+      put_split(sD, r, k, v);
+    }
+    // the tile's gW2 and gW3
+    if (qd >= 2) add_cols(BW_G2 + 8 * (qd + 16 - 18), 0, sum[4]);
+#pragma unroll
+    for (int i = 5; i < 9; ++i) add_cols(BW_G2 + 8 * (qd + 4 * i - 18), 0, sum[i]);
+    if (qd < 2) add_cols(BW_G3 + 8 * qd, 0, sum[9]);
+    publish();
+    if (t == 0) {
+      for (int s = 2; s >= 0; --s)
+        for (int ks = 0; ks < 8; ++ks) {   // gW1^T (M = features of dZ1, N = inputs and the ones, K = rows)
+          const int b = s == 0 && ks >= 4;
+          tcg::mma_f16(taddr + BW_G1 + 144 * b, tcg::sdesc(aD + s * TILE + ks * 4096, 2048, 128),
+                       tcg::sdesc(aX + ks * 4608, 2304, 128), tcg::idesc_bf16(128, 144) | kTA | kTB,
+                       b ? ks > 4 : (s < 2 || ks > 0));
+        }
+      tcg::commit(bar);
+    }
+    wait();   // the next tile overwrites the operands
+    if (!ok) break;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) add_cols(BW_G1 + 8 * (qd + 4 * i), 144, sum[i]);
+    if (qd < 2) add_cols(BW_G1 + 8 * (qd + 16), 144, sum[4]);
   }
-  if (threadIdx.x == 0) atomicAdd(acc, red[0]);
-}
-
-// C (M x N, row-major, ldc) = op(A) op(B) over the k range of this split;
-// op(A)[m][k] = transA ? A[k * lda + m] : A[m * lda + k], same for B with
-// op(B)[k][n].  Partial results of split s go to C + s * M * ldc; a second
-// kernel sums the splits in order (deterministic).
-constexpr int GT = 32;
-__global__ void __launch_bounds__(256)
-gemm_f32(const float* __restrict__ A, int lda, int transA, const float* __restrict__ B, int ldb,
-         int transB, float* __restrict__ C, int ldc, int M, int N, int K, int kchunk) {
-  __shared__ float sA[GT][GT + 1], sB[GT][GT + 1];
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;   // 16 x 16 threads, 2 x 2 outputs each
-  const int m0 = blockIdx.y * GT, n0 = blockIdx.x * GT;
-  const int kb = blockIdx.z * kchunk, ke = min(K, kb + kchunk);
-  float acc[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
-  for (int k0 = kb; k0 < ke; k0 += GT) {
-    for (int i = threadIdx.x; i < GT * GT; i += 256) {
-      const int r = i / GT, c = i % GT;
-      const int m = m0 + r, k = k0 + c;
-      sA[r][c] = (m < M && k < ke) ? (transA ? A[(long long)k * lda + m] : A[(long long)m * lda + k]) : 0.f;
-      const int kk = k0 + r, nn = n0 + c;
-      sB[r][c] = (kk < ke && nn < N) ? (transB ? B[(long long)nn * ldb + kk] : B[(long long)kk * ldb + nn]) : 0.f;
+  // this CTA's sums, in the parameters' layout
+  if (ok) {
+    float* G = part + (size_t)blockIdx.x * NPARAM;
+#pragma unroll
+    for (int i = 0; i < BW_SUMS; ++i) {
+      const int g = qd + 4 * i;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const float v = sum[i][j];
+        if (g < 18) {
+          const int k = 8 * g + j;
+          if (k < IN) G[OFF_W1 + k * HID + r] = v;
+          else if (k == IN) G[OFF_B1 + r] = v;
+        } else if (g < 36) {
+          const int k = 8 * (g - 18) + j;
+          if (k < HID) G[OFF_W2 + k * HID + r] = v;
+          else if (k == HID) G[OFF_B2 + r] = v;
+        }
+      }
+    }
+    // gW3: the three parts' columns c + 3 s lie in two threads' groups (g = 36,
+    // 37); the ninth column passes through shared memory
+    __syncthreads();
+    if (qd == 1) reinterpret_cast<float*>(sX)[r] = sum[9][0];
+    __syncthreads();
+    if (qd == 0) {
+      const float last = reinterpret_cast<float*>(sX)[r];
+#pragma unroll
+      for (int k = 0; k < OUT; ++k)
+        G[OFF_W3 + r * OUT + k] = sum[9][k] + (sum[9][k + 3] + (k + 6 < 8 ? sum[9][(k + 6) & 7] : last));
+    }
+#pragma unroll
+    for (int k = 0; k < OUT; ++k) {
+      float v = qd == 0 ? gb3[k] : 0.f;
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if ((t & 31) == 0) sRed[warp * 8 + k] = v;
+    }
+    if (want_loss) {
+      for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
+      if ((t & 31) == 0 && qd == 0) atomicAdd(acc, loss);
     }
     __syncthreads();
-#pragma unroll 8
-    for (int k = 0; k < GT; ++k) {
-      const float a0 = sA[ty * 2][k], a1 = sA[ty * 2 + 1][k];
-      const float b0 = sB[k][tx * 2], b1 = sB[k][tx * 2 + 1];
-      acc[0][0] = fmaf(a0, b0, acc[0][0]);
-      acc[0][1] = fmaf(a0, b1, acc[0][1]);
-      acc[1][0] = fmaf(a1, b0, acc[1][0]);
-      acc[1][1] = fmaf(a1, b1, acc[1][1]);
-    }
-    __syncthreads();
+    if (t < OUT) G[OFF_B3 + t] = ((sRed[t] + sRed[8 + t]) + sRed[16 + t]) + sRed[24 + t];
+  } else if (!ok && t == 0) {
+    atomicOr(err, 4);
   }
-  float* Cs = C + (long long)blockIdx.z * M * ldc;
-  for (int i = 0; i < 2; ++i)
-    for (int j = 0; j < 2; ++j) {
-      const int m = m0 + ty * 2 + i, nn = n0 + tx * 2 + j;
-      if (m < M && nn < N) Cs[(long long)m * ldc + nn] = acc[i][j];
-    }
+  tcg::fence_before();
+  __syncthreads();
+  if (warp == 0) tcg::dealloc(taddr, 512);
 }
 
-__global__ void sum_splits(const float* __restrict__ part, int splits, int count, float* __restrict__ out) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
-    float s = 0.f;
-    for (int k = 0; k < splits; ++k) s += part[(long long)k * count + i];
-    out[i] = s;
-  }
-}
-
-// column sums of an n x c matrix (bias gradients), two passes
-__global__ void colsum_partial(const float* __restrict__ Z, int n, int c, int rows_per, float* __restrict__ part) {
-  const int col = blockIdx.x * blockDim.x + threadIdx.x;
-  if (col >= c) return;
-  const int r0 = blockIdx.y * rows_per, r1 = min(n, r0 + rows_per);
+// gradients: the CTAs' sums, in four groups of consecutive CTAs, added in order
+__global__ void __launch_bounds__(256) mlp_sum(const float* __restrict__ part, int parts, float* __restrict__ G) {
+  __shared__ float sg[4][64];
+  const int l = threadIdx.x & 63, g = threadIdx.x >> 6, i = blockIdx.x * 64 + l;
+  const int per = (parts + 3) / 4, k1 = min(parts, (g + 1) * per);
   float s = 0.f;
-  for (int r = r0; r < r1; ++r) s += Z[(long long)r * c + col];
-  part[(long long)blockIdx.y * c + col] = s;
-}
-
-__global__ void relu_mask(float* __restrict__ dZ, const float* __restrict__ H, long long count) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < count;
-       i += (long long)gridDim.x * blockDim.x)
-    if (!(H[i] > 0.f)) dZ[i] = 0.f;
+  if (i < NPARAM) {
+#pragma unroll 8
+    for (int k = g * per; k < k1; ++k) s += part[(size_t)k * NPARAM + i];
+  }
+  sg[g][l] = s;
+  __syncthreads();
+  if (g == 0 && i < NPARAM) G[i] = ((sg[0][l] + sg[1][l]) + sg[2][l]) + sg[3][l];
 }
 
 __global__ void adam_kernel(float* __restrict__ P, const float* __restrict__ G, float* __restrict__ m,
@@ -661,8 +918,9 @@ struct MlpImpl {
   float* M2 = nullptr;
   __nv_bfloat16* wt = nullptr;  // transposed bfloat16 weights (W1T | W2T | W3T)
   int max_rows = 0;
-  float *Xr = nullptr, *H1 = nullptr, *H2 = nullptr, *prob = nullptr, *dz3 = nullptr, *dz2 = nullptr,
-        *dz1 = nullptr, *part = nullptr;
+  __nv_bfloat16 *H1 = nullptr, *H2 = nullptr;   // hidden activations of the backward pass's forward
+  float *prob = nullptr, *part = nullptr;       // part: the backward CTAs' sums, [ctas][NPARAM]
+  int ctas = 0;
   double* acc = nullptr;   // loss, weight sum
   int* err = nullptr;      // bit 4: a bounded wait of the tensor-core forward ran out
   int step = 0;
@@ -670,35 +928,14 @@ struct MlpImpl {
   int forward_tc = 1;      // 1: tcgen05 forward (mlp_forward_tc), 0: mma.sync forward
 };
 
-static int gemm(const float* A, int lda, int tA, const float* B, int ldb, int tB, float* C, int M, int N,
-                int K, float* part, size_t part_floats, cudaStream_t st) {
-  int splits = std::max(1, std::min(64, K / 512));
-  while ((size_t)splits * M * N > part_floats && splits > 1) splits /= 2;
-  const int kchunk = ((K + splits - 1) / splits + GT - 1) / GT * GT;
-  splits = (K + kchunk - 1) / kchunk;
-  dim3 grid((N + GT - 1) / GT, (M + GT - 1) / GT, splits);
-  gemm_f32<<<grid, 256, 0, st>>>(A, lda, tA, B, ldb, tB, splits > 1 ? part : C, N, M, N, K, kchunk);
-  if (splits > 1) sum_splits<<<std::min(1024, (M * N + 255) / 256), 256, 0, st>>>(part, splits, M * N, C);
-  SEM_CUDA_TRY(cudaGetLastError());
-  return SEM_OK;
-}
-
-static int colsum(const float* Z, int n, int c, float* out, float* part, cudaStream_t st) {
-  const int rows_per = 1024;
-  const int chunks = (n + rows_per - 1) / rows_per;
-  dim3 grid((c + 127) / 128, chunks);
-  colsum_partial<<<grid, 128, 0, st>>>(Z, n, c, rows_per, part);
-  sum_splits<<<std::max(1, (c + 255) / 256), 256, 0, st>>>(part, chunks, c, out);
-  SEM_CUDA_TRY(cudaGetLastError());
-  return SEM_OK;
-}
-
 int mlp_create(unsigned long long seed, int max_rows, void** out) {
   MlpImpl* m = new MlpImpl();
   m->max_rows = max_rows;
   cudaGetDevice(&m->dev);
   const size_t rows = (size_t)std::max(max_rows, 1);
-  const size_t part_floats = std::max<size_t>(64 * HID * IN, (rows / 1024 + 1) * IN);
+  int nsm = 152;
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, m->dev);
+  m->ctas = (int)std::min<size_t>((rows + 127) / 128, (size_t)nsm);
   cudaError_t e = cudaSuccess;
   auto A = [&](void** p, size_t bytes) { if (e == cudaSuccess) e = cudaMalloc(p, bytes); };
   A((void**)&m->P, NPARAM * 4);
@@ -707,14 +944,10 @@ int mlp_create(unsigned long long seed, int max_rows, void** out) {
   A((void**)&m->M1, NPARAM * 4);
   A((void**)&m->M2, NPARAM * 4);
   A((void**)&m->wt, (size_t)(W1T_SZ + W2T_SZ + W3T_SZ) * 2);
-  A((void**)&m->Xr, rows * IN * 4);
-  A((void**)&m->H1, rows * HID * 4);
-  A((void**)&m->H2, rows * HID * 4);
+  A((void**)&m->H1, rows * HID * 2);
+  A((void**)&m->H2, rows * HID * 2);
   A((void**)&m->prob, rows * OUT * 4);
-  A((void**)&m->dz3, rows * OUT * 4);
-  A((void**)&m->dz2, rows * HID * 4);
-  A((void**)&m->dz1, rows * HID * 4);
-  A((void**)&m->part, part_floats * 4);
+  A((void**)&m->part, (size_t)m->ctas * NPARAM * 4);
   A((void**)&m->acc, 2 * sizeof(double));
   A((void**)&m->err, sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(m->err, 0, sizeof(int));
@@ -725,6 +958,8 @@ int mlp_create(unsigned long long seed, int max_rows, void** out) {
     e = cudaFuncSetAttribute(mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FWD_SMEM);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(mlp_forward_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(mlp_backward_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BW_SMEM);
   if (e == cudaSuccess) {
     // Uniform(-1/sqrt(fan_in), 1/sqrt(fan_in)) weights from splitmix64 of
     // (seed, index), zero biases
@@ -743,8 +978,7 @@ int mlp_create(unsigned long long seed, int max_rows, void** out) {
   }
   if (e != cudaSuccess) {
     std::string msg = cudaGetErrorString(e);
-    void* ps[] = {m->P, m->R, m->G, m->M1, m->M2, m->wt, m->Xr, m->H1, m->H2, m->prob, m->dz3, m->dz2, m->dz1, m->part, m->acc,
-                m->err};
+    void* ps[] = {m->P, m->R, m->G, m->M1, m->M2, m->wt, m->H1, m->H2, m->prob, m->part, m->acc, m->err};
     for (void* p : ps)
       if (p) cudaFree(p);
     delete m;
@@ -759,7 +993,7 @@ int mlp_create(unsigned long long seed, int max_rows, void** out) {
 void mlp_destroy(void* h) {
   MlpImpl* m = (MlpImpl*)h;
   if (!m) return;
-  void* ps[] = {m->P, m->R, m->G, m->M1, m->M2, m->wt, m->Xr, m->H1, m->H2, m->prob, m->dz3, m->dz2, m->dz1, m->part, m->acc};
+  void* ps[] = {m->P, m->R, m->G, m->M1, m->M2, m->wt, m->H1, m->H2, m->prob, m->part, m->acc, m->err};
   for (void* p : ps)
     if (p) cudaFree(p);
   delete m;
@@ -782,7 +1016,7 @@ int mlp_params(void* h, float* host, int set, int which) {
 
 int mlp_param_count() { return NPARAM; }
 
-static void launch_forward(MlpImpl* m, const float* X, int n, float* prob, float* Xr, float* H1, float* H2,
+static void launch_forward(MlpImpl* m, const float* X, int n, float* prob, __nv_bfloat16* H1, __nv_bfloat16* H2,
                            int8_t* flags, cudaStream_t st) {
   if (m->forward_tc) {
     ProfScope ps("mlp_forward_tc", st);
@@ -790,14 +1024,14 @@ static void launch_forward(MlpImpl* m, const float* X, int n, float* prob, float
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     const int tiles = (n + TC_ROWS - 1) / TC_ROWS;
-    mlp_forward_tc<<<std::min(tiles, 2 * nsm), TC_ROWS, TC_SMEM, st>>>(
-        X, n, m->wt, m->wt + W1T_SZ, m->wt + W1T_SZ + W2T_SZ, m->P, prob, Xr, H1, H2, flags, m->err);
+    mlp_forward_tc<<<std::min(tiles, 2 * nsm), TC_T, TC_SMEM, st>>>(
+        X, n, m->wt, m->wt + W1T_SZ, m->wt + W1T_SZ + W2T_SZ, m->P, prob, H1, H2, flags, m->err);
     return;
   }
   const int grid = (n + FWD_ROWS - 1) / FWD_ROWS;
   ProfScope ps("mlp_forward", st);
-  mlp_forward<<<grid, 128, FWD_SMEM, st>>>(X, n, m->wt, m->wt + W1T_SZ, m->wt + W1T_SZ + W2T_SZ, m->P, prob, Xr,
-                                            H1, H2, flags);
+  mlp_forward<<<grid, 128, FWD_SMEM, st>>>(X, n, m->wt, m->wt + W1T_SZ, m->wt + W1T_SZ + W2T_SZ, m->P, prob, H1,
+                                            H2, flags);
 }
 
 int mlp_select_forward(void* h, int tc) {
@@ -820,7 +1054,7 @@ int mlp_status(void* h, int* status, cudaStream_t st) {
 int mlp_forward_api(void* h, const float* X, int n, float* prob, int8_t* flags, cudaStream_t st) {
   MlpImpl* m = (MlpImpl*)h;
   if (n <= 0) return SEM_OK;
-  launch_forward(m, X, n, prob, nullptr, nullptr, nullptr, flags, st);
+  launch_forward(m, X, n, prob, nullptr, nullptr, flags, st);
   SEM_CUDA_TRY(cudaGetLastError());
   return SEM_OK;
 }
@@ -829,27 +1063,14 @@ int mlp_backward_api(void* h, const float* X, const int8_t* y, const float* cw, 
                      cudaStream_t st) {
   MlpImpl* m = (MlpImpl*)h;
   if (n <= 0 || n > m->max_rows) return fail(SEM_ERR_ARG, "row count outside 1..max_rows");
-  const size_t part_floats = std::max<size_t>(64 * HID * IN, ((size_t)m->max_rows / 1024 + 1) * IN);
-  launch_forward(m, X, n, m->prob, m->Xr, m->H1, m->H2, nullptr, st);
+  launch_forward(m, X, n, m->prob, m->H1, m->H2, nullptr, st);
   SEM_CUDA_TRY(cudaMemsetAsync(m->acc, 0, 2 * sizeof(double), st));
-  const int rb = std::min(1024, (n + 255) / 256);
-  mlp_wsum<<<rb, 256, 0, st>>>(y, n, cw[0], cw[1], cw[2], m->acc);
-  mlp_dz3<<<rb, 256, 0, st>>>(m->prob, y, n, cw[0], cw[1], cw[2], m->acc, m->dz3, m->acc);
-  int rc;
+  mlp_wsum<<<std::min(256, (n + 255) / 256), 256, 0, st>>>(y, n, cw[0], cw[1], cw[2], m->acc);
   ProfScope ps("mlp_backward", st);
-  // gW3 = H2r^T dZ3, gb3 = colsum dZ3
-  if ((rc = gemm(m->H2, HID, 1, m->dz3, OUT, 0, m->G + OFF_W3, HID, OUT, n, m->part, part_floats, st))) return rc;
-  if ((rc = colsum(m->dz3, n, OUT, m->G + OFF_B3, m->part, st))) return rc;
-  // dZ2 = (dZ3 W3r^T) * [H2 > 0]
-  if ((rc = gemm(m->dz3, OUT, 0, m->R + OFF_W3, OUT, 1, m->dz2, n, HID, OUT, m->part, part_floats, st))) return rc;
-  relu_mask<<<1024, 256, 0, st>>>(m->dz2, m->H2, (long long)n * HID);
-  if ((rc = gemm(m->H1, HID, 1, m->dz2, HID, 0, m->G + OFF_W2, HID, HID, n, m->part, part_floats, st))) return rc;
-  if ((rc = colsum(m->dz2, n, HID, m->G + OFF_B2, m->part, st))) return rc;
-  // dZ1 = (dZ2 W2r^T) * [H1 > 0]
-  if ((rc = gemm(m->dz2, HID, 0, m->R + OFF_W2, HID, 1, m->dz1, n, HID, HID, m->part, part_floats, st))) return rc;
-  relu_mask<<<1024, 256, 0, st>>>(m->dz1, m->H1, (long long)n * HID);
-  if ((rc = gemm(m->Xr, IN, 1, m->dz1, HID, 0, m->G + OFF_W1, IN, HID, n, m->part, part_floats, st))) return rc;
-  if ((rc = colsum(m->dz1, n, HID, m->G + OFF_B1, m->part, st))) return rc;
+  const int ctas = std::min((n + 127) / 128, m->ctas);
+  mlp_backward_tc<<<ctas, BW_T, BW_SMEM, st>>>(X, y, n, cw[0], cw[1], cw[2], m->prob, m->H1, m->H2, m->R, m->acc,
+                                               loss_host != nullptr, m->part, m->err);
+  mlp_sum<<<(NPARAM + 63) / 64, 256, 0, st>>>(m->part, ctas, m->G);
   SEM_CUDA_TRY(cudaGetLastError());
   if (loss_host) {
     double a[2];
