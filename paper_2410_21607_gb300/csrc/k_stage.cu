@@ -104,6 +104,7 @@ struct VolArgs {
   double g, f, gamma;
   float gf, ff, gammaf;
   float bin[8];         // binomial-series coefficients C(gamma, k), k = 1..7
+  double bin64[10];     // ... k = 1..10
   double geo[kLev][8];
   float geof[kLev][8];
   const float* ref32;
@@ -165,13 +166,35 @@ __device__ __forceinline__ const R* ref_row(const VolArgs& A, int hm, int kz) {
   return refH_of<R>(A) + ((long long)(-1 - hm) * A.NZ + kz) * kRef;
 }
 
-template <typename R> __device__ __forceinline__ R r_log1p(R x);
-template <> __device__ __forceinline__ double r_log1p<double>(double x) { return log1p(x); }
-template <> __device__ __forceinline__ float r_log1p<float>(float x) { return log1pf(x); }
-template <typename R> __device__ __forceinline__ R r_expm1(R x);
-template <> __device__ __forceinline__ double r_expm1<double>(double x) { return expm1(x); }
-template <> __device__ __forceinline__ float r_expm1<float>(float x) { return expm1f(x); }
-
+// 1 / x of a float64: a float32 reciprocal of x's leading bits (relative error
+// e below 2^-21) and one third-order step y (1 + e + e^2), three fused
+// multiply-adds instead of a float64 division on the narrow float64 pipe; the
+// remaining error is that of the last rounding.  Outside float32's comfortable
+// range the division.
+__device__ __forceinline__ double recip_f64(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const int e = (int)((hi >> 20) & 0x7ffu) - 1023;
+  if (e < -100 || e > 100) return 1.0 / x;
+  const float f = __uint_as_float((hi & 0x80000000u) | ((unsigned)(e + 127) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29));
+  const unsigned r = __float_as_uint(__frcp_rn(f));
+  const double y = __hiloint2double((int)((r & 0x80000000u) | ((((r >> 23) & 0xffu) + 896u) << 20) | ((r >> 3) & 0xfffffu)),
+                                    (int)(r << 29));
+  const double d = fma(-x, y, 1.0);
+  return fma(y, fma(d, d, d), y);
+}
+// (1 + x)^gamma - 1 in float64.  For |x| <= 1/32 (perturbations of a few
+// percent) the binomial series sum_{k=1..10} C(gamma, k) x^k in Horner form,
+// whose first dropped term is below 2^-59 of the result: 10 operations on the
+// float64 pipe, where expm1(gamma log1p(x)), taken beyond, costs about 60.
+__device__ __forceinline__ double pow1p_m1_f64(double x, const double* bin, double gam) {
+  if (fabs(x) <= 0.03125) {
+    double s = bin[9];
+#pragma unroll
+    for (int k = 8; k >= 0; --k) s = fma(s, x, bin[k]);
+    return s * x;
+  }
+  return expm1(gam * log1p(x));
+}
 // Gather the 5 fields of local node (ab, kz) of a column (Q row, Sec. 3.1).
 template <int N, typename R>
 __device__ __forceinline__ void gather_node(const VolArgs& A, int hm, int kz, R v[kFields]) {
@@ -278,11 +301,11 @@ volume_column(const VolArgs A) {
       const R p0 = rf[2], rho0 = rf[3], rt0 = rf[4], inv_rt0 = rf[6];
       const R rp = v[0];
       const R rho = rho0 + rp;
-      const R inv = (R)1 / rho;
+      const R inv = recip_f64(rho);
       if (EQ == 0) {
         const R U = v[1], V = v[2], W = v[3], Tp = v[4];
         const R u = U * inv, vv = V * inv, w = W * inv;
-        const R pp = p0 * r_expm1<R>(gam * r_log1p<R>(Tp * inv_rt0));
+        const R pp = p0 * pow1p_m1_f64(Tp * inv_rt0, A.bin64, gam);
         const R rt = rt0 + Tp;
         const R ax = wj * wc * sx, ay = wi * wc * sy, az = wi * wj * sz;
         if (!WARP) {
@@ -309,7 +332,7 @@ volume_column(const VolArgs A) {
         const R u = v[1], vv = v[2], w = v[3], thp = v[4];
         const R th0 = rf[0];
         const R rtp = rho0 * thp + rp * (th0 + thp);
-        const R pp = p0 * r_expm1<R>(gam * r_log1p<R>(rtp * inv_rt0));
+        const R pp = p0 * pow1p_m1_f64(rtp * inv_rt0, A.bin64, gam);
         const R ax = wj * wc * sx, ay = wi * wc * sy, az = wi * wj * sz;
         sF[0][t] = rho * u * ax;
         sF[1][t] = rho * vv * ay;
@@ -626,22 +649,243 @@ __global__ void __launch_bounds__(256) mirror_kernel(const double* q, float* q32
     q32[i] = d2f_bits(q[i]);
 }
 
-// The float64 form's element kernel (both sets, box or warped layers); the
-// mixed form runs the line-exchange kernels of the variant table instead.
-template <int N, int EQ>
-static void launch_volume(const VolArgs& A, cudaStream_t st) {
-  constexpr int P = (N + 1) * (N + 1) * (N + 1);
-  constexpr int nt = (P + 31) / 32 * 32;
-  ProfScope ps("volume_fp64", st);
-  if (A.metric)
-    volume_column<N, EQ, double, true><<<A.Ncol, nt, 0, st>>>(A);
-  else
-    volume_column<N, EQ, double><<<A.Ncol, nt, 0, st>>>(A);
+// Float64 form, conservative set, box meshes.  The float64 pipe (1/64 of the
+// float32 rate) is what the element pass costs, so the kernel is laid out to
+// issue as few float64 instructions per node as it can; moving values through
+// shared memory is free beside them.
+//   - A level that two layers share is worked on once: its weak x and y terms
+//     take the sum of both layers' weights (the layer thickness enters them as
+//     a factor), so a column of nz layers has nz N + 1 levels of fluxes instead
+//     of nz (N + 1).
+//   - The contractions run on lines and planes with compile-time
+//     coefficients, which drops the zeros on the derivative matrix's diagonal.
+//   - Weights are applied per level and per node, not per flux component.
+// One CTA per column, KL layers at a time: (A) a thread per node forms the
+// weighted fluxes; (B) a thread per (field, level) contracts x and y over the
+// plane's (N+1)^2 nodes in registers; (C) a thread per (field, node, layer)
+// contracts z and adds it, its top value going to the layer above; (D) Coriolis
+// and buoyancy are added and the column residual is stored.  Lanes run along z
+// throughout.  The level above a chunk is carried into the next one.
+// 32x32x16, N = 4: 471 us, float64 pipe 81 % busy (1024 columns are 3.4 waves of
+// two CTAs per SM); volume_column, a thread per element node, took 652 us (90 %).
+template <int N> struct ChunkCfg;
+template <> struct ChunkCfg<2> { static constexpr int KL = 16; };
+template <> struct ChunkCfg<3> { static constexpr int KL = 8; };
+template <> struct ChunkCfg<4> { static constexpr int KL = 8; };
+template <> struct ChunkCfg<5> { static constexpr int KL = 4; };
+template <> struct ChunkCfg<6> { static constexpr int KL = 2; };
+constexpr int kChunkThreads = 256;
+template <int N> struct ChunkSmem {   // in doubles
+  static constexpr int Nq = (N + 1) * (N + 1), KL = ChunkCfg<N>::KL, LD = KL * N + 1;
+  static constexpr int F = 5 * Nq * LD;              // one flux buffer [5][Nq][LD]
+  static constexpr int TOP = 3 * F;                  // z part of each layer's top level [5][Nq][KL]
+  static constexpr int CAR = TOP + 5 * Nq * KL;      // ... of the chunk's last layer [5][Nq]
+  static constexpr int LEV = CAR + 5 * Nq;           // per level: sx W, sy W, J W f, J W g
+  static constexpr int AB = LEV + 4 * LD;            // per node: w_j, w_i, w_i w_j sz, w_i w_j
+  static constexpr int HM = AB + 4 * Nq;             // column map (int)
+  static constexpr int TOTAL = HM + (Nq + 1) / 2;
+};
+
+template <int N>
+__global__ void __launch_bounds__(kChunkThreads, N == 3 || N == 2 ? 3 : 2)
+volume_chunk(const VolArgs A) {
+  using L = ChunkSmem<N>;
+  constexpr int n1 = N + 1, Nq = n1 * n1, KL = L::KL, LD = L::LD, T = kChunkThreads;
+  extern __shared__ __align__(16) double sm64[];
+  double *sX = sm64, *sY = sX + L::F, *sZ = sY + L::F, *sTop = sm64 + L::TOP, *sCar = sm64 + L::CAR;
+  double *sLev = sm64 + L::LEV, *sAb = sm64 + L::AB;
+  int* s_hm = reinterpret_cast<int*>(sm64 + L::HM);
+  const int col = blockIdx.x, t = threadIdx.x;
+  const double* geo = A.geo[A.col_level[col]];
+  for (int ab = t; ab < Nq; ab += T) {
+    s_hm[ab] = A.hmap[(long long)col * Nq + ab];
+    const double wi = c_w[N][ab % n1], wj = c_w[N][ab / n1];
+    sAb[4 * ab + 0] = wj;
+    sAb[4 * ab + 1] = wi;
+    sAb[4 * ab + 2] = wi * wj * geo[6];
+    sAb[4 * ab + 3] = wi * wj;
+  }
+  const double* q = (const double*)A.q;
+  double* rc = (double*)A.rc;
+  for (int k0 = 0; k0 < A.nz; k0 += KL) {
+    const int kl = min(KL, A.nz - k0), lv = kl * N;   // levels 0 .. lv of the chunk; lv belongs to the next one
+    const bool last = k0 + kl == A.nz;
+    const int own = last ? lv + 1 : lv;               // levels whose residual this chunk completes
+    const int beg = k0 == 0 ? 0 : 1;                  // level 0 came with the previous chunk
+    __syncthreads();
+    for (int l = t; l <= lv; l += T) {
+      const int kz = k0 * N + l, k = kz / N, c = kz - k * N;
+      double W = 0.0;
+      if (c > 0) {
+        W = c_w[N][c] * A.hzk[k];
+      } else {
+        if (k < A.nz) W = c_w[N][0] * A.hzk[k];
+        if (k > 0) W = fma(c_w[N][N], A.hzk[k - 1], W);
+      }
+      sLev[4 * l + 0] = geo[4] * W;
+      sLev[4 * l + 1] = geo[5] * W;
+      sLev[4 * l + 2] = geo[3] * W * A.f;
+      sLev[4 * l + 3] = geo[3] * W * A.g;
+    }
+    __syncthreads();
+    // (A) fluxes
+    const int nl = lv + 1 - beg;
+    for (int it = t; it < Nq * nl; it += T) {
+      const int ab = it / nl, l = it - ab * nl + beg, kz = k0 * N + l;
+      double v[kFields];
+      gather_node<N, double>(A, s_hm[ab], kz, v);
+      const double* rf = A.ref + (long long)kz * kRef;
+      const double p0 = __ldg(rf + 2), rho0 = __ldg(rf + 3), rt0 = __ldg(rf + 4), irt0 = __ldg(rf + 6);
+      const double U = v[1], V = v[2], W = v[3];
+      const double inv = recip_f64(rho0 + v[0]);
+      const double pp = p0 * pow1p_m1_f64(v[4] * irt0, A.bin64, A.gamma);
+      const double rt = rt0 + v[4];
+      const double ax = sLev[4 * l] * sAb[4 * ab], ay = sLev[4 * l + 1] * sAb[4 * ab + 1], az = sAb[4 * ab + 2];
+      const double ux = U * inv * ax, vy = V * inv * ay, wz = W * inv * az;
+      double* x = sX + ab * LD + l;
+      double* y = sY + ab * LD + l;
+      double* z = sZ + ab * LD + l;
+      constexpr int FS = Nq * LD;
+      x[0] = U * ax; x[FS] = fma(U, ux, pp * ax); x[2 * FS] = V * ux; x[3 * FS] = W * ux; x[4 * FS] = rt * ux;
+      y[0] = V * ay; y[FS] = U * vy; y[2 * FS] = fma(V, vy, pp * ay); y[3 * FS] = W * vy; y[4 * FS] = rt * vy;
+      z[0] = W * az; z[FS] = U * wz; z[2 * FS] = V * wz; z[3 * FS] = fma(W, wz, pp * az); z[4 * FS] = rt * wz;
+    }
+    __syncthreads();
+    // (B) x and y on the planes that this chunk completes, over sX
+    for (int it = t; it < kFields * own; it += T) {
+      const int f = it / own, l = it - f * own;
+      double* x = sX + f * Nq * LD + l;
+      const double* y = sY + f * Nq * LD + l;
+      double acc[Nq];
+#pragma unroll
+      for (int j = 0; j < n1; ++j) {
+        double F[n1];
+#pragma unroll
+        for (int m = 0; m < n1; ++m) F[m] = x[(m + n1 * j) * LD];
+#pragma unroll
+        for (int i = 0; i < n1; ++i) {
+          double a = 0.0;
+          bool any = false;
+#pragma unroll
+          for (int m = 0; m < n1; ++m)
+            if (!(i == m && i > 0 && i < N)) {
+              a = any ? fma(c_Dw[N][i * n1 + m], F[m], a) : c_Dw[N][i * n1 + m] * F[m];
+              any = true;
+            }
+          acc[i + n1 * j] = a;
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < n1; ++i) {
+        double F[n1];
+#pragma unroll
+        for (int m = 0; m < n1; ++m) F[m] = y[(i + n1 * m) * LD];
+#pragma unroll
+        for (int j = 0; j < n1; ++j)
+#pragma unroll
+          for (int m = 0; m < n1; ++m)
+            if (!(j == m && j > 0 && j < N)) acc[i + n1 * j] = fma(c_Dw[N][j * n1 + m], F[m], acc[i + n1 * j]);
+      }
+#pragma unroll
+      for (int ab = 0; ab < Nq; ++ab) x[ab * LD] = acc[ab];
+    }
+    __syncthreads();
+    // (C) z on the layers' lines
+    for (int it = t; it < kFields * Nq * kl; it += T) {
+      const int fa = it / kl, k = it - fa * kl;
+      const double* z = sZ + fa * LD + k * N;
+      double* x = sX + fa * LD + k * N;
+      double F[n1];
+#pragma unroll
+      for (int m = 0; m < n1; ++m) F[m] = z[m];
+#pragma unroll
+      for (int c = 0; c < n1; ++c) {
+        double a = c < N ? x[c] : 0.0;
+#pragma unroll
+        for (int m = 0; m < n1; ++m)
+          if (!(c == m && c > 0 && c < N)) a = fma(c_Dw[N][c * n1 + m], F[m], a);
+        if (c < N) x[c] = a;
+        else sTop[fa * KL + k] = a;
+      }
+    }
+    __syncthreads();
+    // (D) faces between layers, Coriolis and buoyancy, store
+    for (int it = t; it < kFields * Nq * own; it += T) {
+      const int fa = it / own, l = it - fa * own, f = fa / Nq, ab = fa - f * Nq, kz = k0 * N + l;
+      const int k = l / N;
+      double r;
+      if (l == lv) r = sX[fa * LD + l] + sTop[fa * KL + kl - 1];   // the lid
+      else {
+        r = sX[fa * LD + l];
+        if (l == k * N && (k > 0 || k0 > 0)) r += k > 0 ? sTop[fa * KL + k - 1] : sCar[fa];
+      }
+      if (f >= 1 && f <= 3) {
+        const int src = f == 1 ? 2 : (f == 2 ? 1 : 0);
+        const int hm = s_hm[ab];
+        double v;
+        if (hm >= 0) {
+          v = __ldg(q + (long long)src * A.NG + (long long)hm * A.NZ + kz);
+        } else {
+          const int h = -1 - hm;
+          v = 0.0;
+          for (int m = 0; m < n1; ++m)
+            v += __ldg((const double*)A.hang_w + h * n1 + m) *
+                 __ldg(q + (long long)src * A.NG + (long long)__ldg(A.hang_h + h * n1 + m) * A.NZ + kz);
+        }
+        const double c = sLev[4 * l + (f == 3 ? 3 : 2)] * sAb[4 * ab + 3];
+        r = f == 1 ? fma(c, v, r) : fma(-c, v, r);
+      }
+      rc[((long long)col * Nq * kFields + ab * kFields + f) * A.NZr + kz] = r;
+    }
+    __syncthreads();
+    if (!last) {
+      // the level above: its fluxes, and the z part of the layer below it
+      for (int fa = t; fa < kFields * Nq; fa += T) {
+        sX[fa * LD] = sX[fa * LD + lv];
+        sY[fa * LD] = sY[fa * LD + lv];
+        sZ[fa * LD] = sZ[fa * LD + lv];
+        sCar[fa] = sTop[fa * KL + kl - 1];
+      }
+    }
+  }
 }
 
 template <int N>
-static void launch_volume_fp64(const VolArgs& A, int eq, cudaStream_t st) {
-  if (eq == 0) launch_volume<N, 0>(A, st); else launch_volume<N, 1>(A, st);
+static int launch_chunk(const VolArgs& A, cudaStream_t st) {
+  constexpr size_t sm = sizeof(double) * ChunkSmem<N>::TOTAL;
+  static DeviceOnce attr;
+  const int rc = device_once(attr, [&] {
+    SEM_CUDA_TRY(cudaFuncSetAttribute(volume_chunk<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    return SEM_OK;
+  });
+  if (rc) return rc;
+  ProfScope ps("volume_fp64", st);
+  volume_chunk<N><<<A.Ncol, kChunkThreads, sm, st>>>(A);
+  return SEM_OK;
+}
+
+// The float64 form's other element kernels (the paper's set, warped layers); the
+// mixed form runs the line-exchange kernels of the variant table instead.
+template <int N, int EQ>
+static void launch_volume_warp(const VolArgs& A, cudaStream_t st) {
+  constexpr int P = (N + 1) * (N + 1) * (N + 1);
+  ProfScope ps("volume_fp64", st);
+  volume_column<N, EQ, double, true><<<A.Ncol, (P + 31) / 32 * 32, 0, st>>>(A);
+}
+template <int N, int EQ>
+static void launch_volume(const VolArgs& A, cudaStream_t st) {
+  if (A.metric) return launch_volume_warp<N, EQ>(A, st);
+  constexpr int P = (N + 1) * (N + 1) * (N + 1);
+  ProfScope ps("volume_fp64", st);
+  volume_column<N, EQ, double><<<A.Ncol, (P + 31) / 32 * 32, 0, st>>>(A);
+}
+
+template <int N>
+static int launch_volume_fp64(const VolArgs& A, int eq, cudaStream_t st) {
+  if (eq == 0 && !A.metric) return launch_chunk<N>(A, st);
+  if (eq == 0) launch_volume_warp<N, 0>(A, st);
+  else launch_volume<N, 1>(A, st);
+  return SEM_OK;
 }
 
 // ---------------------------------------------------------------------------
@@ -2086,9 +2330,10 @@ static VolArgs make_vol_args(Mesh& m, const sem_params& p, const void* q, bool m
   A.gammaf = (float)A.gamma;
   {
     double cb = 1.0;
-    for (int k = 1; k <= 7; ++k) {
+    for (int k = 1; k <= 10; ++k) {
       cb *= (A.gamma - (k - 1)) / k;
-      A.bin[k - 1] = (float)cb;
+      A.bin64[k - 1] = cb;
+      if (k <= 7) A.bin[k - 1] = (float)cb;
     }
     A.bin[7] = 0.f;
   }
@@ -2876,13 +3121,14 @@ int launch_rhs_stage(Mesh& m, const sem_params& p, const StageArgs& s, cudaStrea
   } else if (mixed) {
     if ((rc = launch_nc_n(A, m.N, m.nz, st, m.nc_variant))) return rc;
   } else switch (m.N) {
-    case 2: launch_volume_fp64<2>(A, eq, st); break;
-    case 3: launch_volume_fp64<3>(A, eq, st); break;
-    case 4: launch_volume_fp64<4>(A, eq, st); break;
-    case 5: launch_volume_fp64<5>(A, eq, st); break;
-    case 6: launch_volume_fp64<6>(A, eq, st); break;
+    case 2: rc = launch_volume_fp64<2>(A, eq, st); break;
+    case 3: rc = launch_volume_fp64<3>(A, eq, st); break;
+    case 4: rc = launch_volume_fp64<4>(A, eq, st); break;
+    case 5: rc = launch_volume_fp64<5>(A, eq, st); break;
+    case 6: rc = launch_volume_fp64<6>(A, eq, st); break;
     default: return fail(SEM_ERR_UNSUPPORTED, "order N not compiled");
   }
+  if (rc) return rc;
   SEM_CUDA_TRY(cudaGetLastError());
   if (physics_on(p) &&
       (rc = launch_physics(m, p, mixed ? (const void*)qs32 : (const void*)s.qs, mixed, s.scratch, s.time, st,
