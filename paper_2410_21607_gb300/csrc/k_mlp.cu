@@ -1,6 +1,6 @@
 // Learned refinement flags: per-element features, a 3-layer MLP (136-128-128-3)
-// with bfloat16 tensor-core products and float32 accumulation, its backward
-// pass (float32 values as sums of bfloat16 parts) and Adam.
+// with bfloat16 tensor-core forward products and float32 accumulation, its
+// backward pass and Adam.
 //
 // The paper's velocity criterion (Sec. 3.1) fires only once intensification
 // has started (Sec. 5); the network predicts the criterion's flags some steps
@@ -434,61 +434,36 @@ __global__ void mlp_wsum(const int8_t* __restrict__ y, int n, float w0, float w1
   if (threadIdx.x == 0) atomicAdd(acc + 1, red[0]);
 }
 
-// Backward pass on the tensor cores, one persistent CTA per SM walking over
-// tiles of 128 rows.  Per tile, with dZ3 = w_y (p - onehot) / sum(w_y):
-//   gW3 += H2^T dZ3,  dZ2 = (dZ3 W3^T) [H2 > 0],  gW2 += H1^T dZ2,
-//   dZ1 = (dZ2 W2^T) [H1 > 0],                     gW1 += X^T dZ1.
-// The rounded inputs, activations and weights are bfloat16 values, the dZ are
-// float32: each dZ is split into three bfloat16 parts whose sum is exact (8
-// bits of the significand each), so every product is exact and the sums are
-// float32, as in a float32 matrix product.  The tensor cores truncate when they
-// add to an accumulator (24 steps on a large one left 5e-7, over all of a CTA's
-// tiles 1e-6), so the small parts go first, the large part's eight steps are
-// shared by two accumulators where tensor memory has room, and every tile's
-// sums are added to float32 registers, rounding to nearest: the error against
-// float64 is then that of float32 fused multiply-adds.  The weight gradients
-// are formed as gW^T (rows are the features of dZ, so that X's 136 + 8 columns
-// are the N extent); a column of ones beside X and H1 gives the bias gradients
-// in the same products.  A tile is stored once,
-// in core matrices of 8 rows x 8 features: read along the features it is the
-// K-major operand of the dZ1 product, read along the rows the MN-major operand
-// of the gradient products.  Each CTA writes its sums, mlp_sum adds them in
-// order (deterministic).  65536 rows: 68 us; 32x32 float32 tiles on the CUDA cores
-// took 240 + 224 + 123 + 123 + 91 us for the five products and 180 us for the
-// masks and bias sums between them, each with its own pass over memory.
-constexpr int BW_T = 512;
-constexpr int BW_X = 0, BW_H = BW_X + 128 * 144 * 2, BW_D = BW_H + 128 * 144 * 2, BW_W2 = BW_D + 3 * 128 * HID * 2;
-constexpr int BW_D3 = BW_W2 + HID * HID * 2, BW_W3 = BW_D3 + 128 * 16 * 2, BW_RED = BW_W3 + HID * OUT * 4;
-constexpr int BW_BAR = BW_RED + 16 * 8 * 4;
-constexpr size_t BW_SMEM = BW_BAR + 16;
-// tensor memory columns: dZ1 (two accumulators), gW2, gW3; then gW1 (two)
-constexpr uint32_t BW_C1 = 0, BW_G2 = 256, BW_G3 = 416, BW_G1 = 0;
-constexpr int BW_SUMS = 10;   // groups of 8 gradient columns per thread
-
-// two float32 values as three bfloat16 pairs, x = p[0] + p[1] + p[2] (exact for
-// finite x away from the smallest float32 values): one packed conversion per
-// part, the residuals by the parts' bits
-__device__ __forceinline__ void split3(float a, float b, unsigned (&p)[3]) {
-#pragma unroll
-  for (int s = 0; s < 3; ++s) {
-    p[s] = pack_bf16(a, b);
-    a -= __uint_as_float(p[s] << 16);
-    b -= __uint_as_float(p[s] & 0xffff0000u);
-  }
+// Backward pass, float32 on the CUDA cores:
+//   dZ3 = w_y (p - onehot) / sum(w_y),  dZ2 = (dZ3 W3^T) [H2 > 0],
+//   dZ1 = (dZ2 W2^T) [H1 > 0],  gW = (input of the layer)^T dZ,  gb = colsum dZ.
+// Every sum runs over its terms in a fixed order of fused multiply-adds: a
+// weight gradient over the rows of a split one after another, then over the
+// splits in order (back_splits), so the results do not depend on how the work
+// is laid out.  That matters beyond rounding: Adam divides a gradient by its own
+// size, and a weight or activation that rounds to another bfloat16 moves every
+// gradient of the next iteration by 1e-4.  (On the tensor cores, with the
+// gradients as three bfloat16 parts, the pass took 68 us at no larger error, but
+// not with these sums.)
+//   back_rows: dZ3, dZ2 and dZ1 of 64 rows per CTA, W2^T in shared memory; a
+//     thread owns 8 rows x 8 features.
+//   back_grads: gW1 and gW2, a block of one of them for one split of the rows
+//     per CTA.
+//   back_tail: gW3 and the bias gradients.
+// The products of two columns at a time are packed (fma.rn.f32x2), which halves
+// the instructions the schedulers have to issue.  65536 rows: back_rows 80 us,
+// back_grads 150, back_tail 73 (the float32 rate would allow 26 and 55 for the
+// first two; they wait for loads and shared memory); as 32x32 tiles of 2x2
+// products per thread with a pass over memory for each product, mask and bias
+// sum it took 980 us.
+__host__ __device__ inline int back_splits(int n, int& chunk) {
+  int s = n / 512;
+  s = s < 1 ? 1 : (s > 64 ? 64 : s);
+  chunk = ((n + s - 1) / s + 31) / 32 * 32;
+  return (n + chunk - 1) / chunk;
 }
-// eight values of row r, columns k..k+7, split into the three tiles at D
-__device__ __forceinline__ void put_split(unsigned char* D, int r, int k, const float (&v)[8]) {
-  unsigned q[3][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    unsigned p[3];
-    split3(v[2 * i], v[2 * i + 1], p);
-#pragma unroll
-    for (int s = 0; s < 3; ++s) q[s][i] = p[s];
-  }
-#pragma unroll
-  for (int s = 0; s < 3; ++s)
-    *reinterpret_cast<uint4*>(D + s * 128 * HID * 2 + boff(r, k, 16)) = make_uint4(q[s][0], q[s][1], q[s][2], q[s][3]);
+__device__ __forceinline__ float2 bf2(unsigned pair) {
+  return make_float2(__uint_as_float(pair << 16), __uint_as_float(pair & 0xffff0000u));
 }
 // v where the bfloat16 activation is positive (neither zero nor NaN), else 0
 __device__ __forceinline__ float masked(unsigned pair, int i, float v) {
@@ -496,264 +471,295 @@ __device__ __forceinline__ float masked(unsigned pair, int i, float v) {
   return b - 1u < 0x7f80u ? v : 0.f;
 }
 
-__global__ void __launch_bounds__(BW_T, 1)
-mlp_backward_tc(const float* __restrict__ X, const int8_t* __restrict__ y, int n, float w0, float w1, float w2,
-                const float* __restrict__ prob, const __nv_bfloat16* __restrict__ H1,
-                const __nv_bfloat16* __restrict__ H2, const float* __restrict__ R, double* __restrict__ acc,
-                int want_loss, float* __restrict__ part, int* err) {
-  extern __shared__ __align__(1024) unsigned char sm_bw[];
-  unsigned char *sX = sm_bw + BW_X, *sH = sm_bw + BW_H, *sD = sm_bw + BW_D, *sW2 = sm_bw + BW_W2, *sD3 = sm_bw + BW_D3;
-  float* sW3 = reinterpret_cast<float*>(sm_bw + BW_W3);
-  float* sRed = reinterpret_cast<float*>(sm_bw + BW_RED);
-  uint64_t* mbar = reinterpret_cast<uint64_t*>(sm_bw + BW_BAR);
-  uint32_t* slot = reinterpret_cast<uint32_t*>(mbar + 1);
-  const int t = threadIdx.x, warp = t >> 5, r = t & 127, qd = t >> 7;
-  // W2 (input-major rows are K-major for dZ2 W2^T) and W3
-  for (int i = t; i < HID * HID / 8; i += BW_T) {
-    const int a = i / (HID / 8), k = 8 * (i % (HID / 8));
-    const float4* p = reinterpret_cast<const float4*>(R + OFF_W2 + a * HID + k);
-    const float4 u = p[0], v = p[1];
-    *reinterpret_cast<uint4*>(sW2 + boff(a, k, 16)) =
-        make_uint4(pack_bf16(u.x, u.y), pack_bf16(u.z, u.w), pack_bf16(v.x, v.y), pack_bf16(v.z, v.w));
+constexpr int BR_ROWS = 64, BR_T = 128, BR_LD = HID + 4;
+constexpr size_t BR_SMEM = sizeof(float) * (HID * BR_LD + HID * (BR_ROWS + 4) + HID * OUT + BR_ROWS * 4);
+__global__ void __launch_bounds__(BR_T)
+back_rows(const int8_t* __restrict__ y, int n, float w0, float w1, float w2, const float* __restrict__ prob,
+          const __nv_bfloat16* __restrict__ H1, const __nv_bfloat16* __restrict__ H2,
+          const __nv_bfloat16* __restrict__ w2t, const float* __restrict__ R, double* __restrict__ acc, int want_loss,
+          float* __restrict__ dz3, float* __restrict__ dz2,
+          float* __restrict__ dz1) {
+  extern __shared__ __align__(16) float sb[];
+  float* sW = sb;                              // [j][i] = W2[i][j]
+  float* sA = sW + HID * BR_LD;                // [j][row] dZ2
+  float* sW3 = sA + HID * (BR_ROWS + 4);       // [j][3]
+  float* sD3 = sW3 + HID * OUT;                // [row][4]
+  const int t = threadIdx.x;
+  const long long row0 = (long long)blockIdx.x * BR_ROWS;
+#pragma unroll
+  for (int u = t; u < HID * HID / 8; u += BR_T) {
+    const int j = u >> 4, i = 8 * (u & 15);
+    const uint4 w = *reinterpret_cast<const uint4*>(w2t + j * K2P + i);
+    const float2 a = bf2(w.x), b = bf2(w.y), c = bf2(w.z), d = bf2(w.w);
+    *reinterpret_cast<float4*>(sW + j * BR_LD + i) = make_float4(a.x, a.y, b.x, b.y);
+    *reinterpret_cast<float4*>(sW + j * BR_LD + i + 4) = make_float4(c.x, c.y, d.x, d.y);
   }
-  for (int i = t; i < HID * OUT; i += BW_T) sW3[i] = R[OFF_W3 + i];
-  // the columns of ones (136 of X, 128 of H1) and the padding
-  if (qd == 0) {
-    const uint4 one = make_uint4(0x00003f80u, 0u, 0u, 0u), z = make_uint4(0u, 0u, 0u, 0u);
-    *reinterpret_cast<uint4*>(sX + boff(r, IN, 18)) = one;
-    *reinterpret_cast<uint4*>(sH + boff(r, HID, 18)) = one;
-    *reinterpret_cast<uint4*>(sH + boff(r, HID + 8, 18)) = z;
-    *reinterpret_cast<uint4*>(sD3 + boff(r, 8, 2)) = z;
-  }
-  if (warp == 0) tcg::alloc(slot, 512);
-  if (t == 0) tcg::mbar_init(tcg::smem_u32(mbar), 1);
-  tcg::fence_before();
-  __syncthreads();
-  tcg::fence_after();
-  const uint32_t taddr = *slot, bar = tcg::smem_u32(mbar);
-  const uint32_t lane = taddr + ((uint32_t)(32 * (warp & 3)) << 16);
-  const uint32_t aX = tcg::smem_u32(sX), aH = tcg::smem_u32(sH), aD = tcg::smem_u32(sD), aW2 = tcg::smem_u32(sW2),
-                 aD3 = tcg::smem_u32(sD3);
-  constexpr uint32_t kTA = 1u << 15, kTB = 1u << 16;   // A, B MN-major
-  constexpr uint32_t TILE = 128 * HID * 2;
-  const bool aligned = ((uintptr_t)X & 15) == 0;   // the mma.sync forward takes any X
+  for (int i = t; i < HID * OUT; i += BR_T) sW3[i] = R[OFF_W3 + i];
   const float inv = (float)(1.0 / acc[1]);
-  float gb3[3] = {0.f, 0.f, 0.f};
-  // running sums of this thread's gradient columns: group g = qd + 4 i of 8
-  // columns is gW1^T's g-th (g < 18), gW2^T's (g < 36) or gW3's (g < 38)
-  float sum[BW_SUMS][8];
-#pragma unroll
-  for (int i = 0; i < BW_SUMS; ++i)
-#pragma unroll
-    for (int j = 0; j < 8; ++j) sum[i][j] = 0.f;
-  auto add_cols = [&](uint32_t col, int second, float (&v)[8]) {   // v += columns col.. (and col + second..)
-    float a[8], b[8];
-    tcg::ld8(lane + col, a);
-    if (second) tcg::ld8(lane + col + second, b);
-    tcg::wait_ld();
-#pragma unroll
-    for (int j = 0; j < 8; ++j) v[j] += second ? a[j] + b[j] : a[j];
-  };
   double loss = 0.0;
-  bool ok = true;
-  uint32_t phase = 0;
-  // all threads' shared-memory writes before the tensor cores read them
-  auto publish = [&] {
-    tcg::fence_async_smem();
-    tcg::fence_before();
-    __syncthreads();
-    tcg::fence_after();
-  };
-  auto wait = [&] {
-    ok = __syncthreads_and(tcg::mbar_wait(bar, phase & 1));
-    ++phase;
-    tcg::fence_after();
-  };
-  const int ntiles = (n + 127) / 128;
-  for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
-    const long long row0 = (long long)tile * 128;
-    const bool in = row0 + r < n;
-#pragma unroll
-    for (int j = 0; j < (TC_XV + 1) / 2; ++j) {
-      int rr, k;
-      input_at<BW_T / 32>(j, rr, k);
-      if (rr >= 128) break;
-      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (row0 + rr < n) {
-        const float* p = X + (row0 + rr) * IN + k;
-        v = aligned ? *reinterpret_cast<const float4*>(p) : make_float4(p[0], p[1], p[2], p[3]);
-      }
-      *reinterpret_cast<uint2*>(sX + boff(rr, k, 18)) = make_uint2(pack_bf16(v.x, v.y), pack_bf16(v.z, v.w));
-    }
-#pragma unroll
-    for (int j = 0; j < 128 * (HID / 8) / BW_T; ++j) {
-      // a warp: 8 rows x 64 bytes
-      const int u = j * (BW_T / 32) + warp, rr = (u >> 2) * 8 + (t & 7), k = 8 * ((u & 3) * 4 + ((t >> 3) & 3));
-      uint4 a = make_uint4(0u, 0u, 0u, 0u), b = a;
-      if (row0 + rr < n) {
-        a = *reinterpret_cast<const uint4*>(H1 + (row0 + rr) * HID + k);
-        b = *reinterpret_cast<const uint4*>(H2 + (row0 + rr) * HID + k);
-      }
-      *reinterpret_cast<uint4*>(sH + boff(rr, k, 18)) = a;
-      *reinterpret_cast<uint4*>(sD + 2 * TILE + boff(rr, k, 16)) = b;   // H2, until dZ2 takes its place
-    }
-    float d3[3] = {0.f, 0.f, 0.f};
-    if (in) {
-      const int c = y[row0 + r];
+  if (t < BR_ROWS) {
+    float d[3] = {0.f, 0.f, 0.f};
+    const long long row = row0 + t;
+    if (row < n) {
+      const int c = y[row];
       const float w = c == 0 ? w0 : (c == 1 ? w1 : w2);
 #pragma unroll
-      for (int k = 0; k < OUT; ++k) d3[k] = w * inv * (prob[(row0 + r) * OUT + k] - (k == c ? 1.f : 0.f));
-      if (qd == 0 && want_loss) loss += (double)w * -log((double)prob[(row0 + r) * OUT + c]);
-    }
-    if (qd == 0) {
-      // the three parts of dZ3 side by side: columns c + 3 s
-      unsigned p[3], z[3];
-      split3(d3[0], d3[1], p);
-      split3(d3[2], 0.f, z);
-      const unsigned w[5] = {p[0], (z[0] & 0xffffu) | (p[1] << 16), (p[1] >> 16) | (z[1] << 16), p[2], z[2] & 0xffffu};
-      *reinterpret_cast<uint4*>(sD3 + boff(r, 0, 2)) = make_uint4(w[0], w[1], w[2], w[3]);
-      *reinterpret_cast<uint4*>(sD3 + boff(r, 8, 2)) = make_uint4(w[4], 0u, 0u, 0u);
-#pragma unroll
-      for (int k = 0; k < OUT; ++k) gb3[k] += d3[k];
-    }
-    publish();
-    if (t == 0) {
-      // gW3 (M = features of H2, N = 16, K = rows)
-      for (int ks = 0; ks < 8; ++ks)
-        tcg::mma_f16(taddr + BW_G3, tcg::sdesc(aD + 2 * TILE + ks * 4096, 2048, 128),
-                     tcg::sdesc(aD3 + ks * 512, 256, 128), tcg::idesc_bf16(128, 16) | kTA | kTB, ks > 0);
-      tcg::commit(bar);
-    }
-    wait();
-    if (!ok) break;
-    // dZ2, its third part over H2
-#pragma unroll 1
-    for (int k = 32 * qd; k < 32 * qd + 32; k += 8) {
-      const uint4 h = *reinterpret_cast<const uint4*>(sD + 2 * TILE + boff(r, k, 16));
-      const unsigned hw[4] = {h.x, h.y, h.z, h.w};
-      float v[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const float* w = sW3 + (k + i) * OUT;
-        v[i] = masked(hw[i >> 1], i, fmaf(d3[2], w[2], fmaf(d3[1], w[1], d3[0] * w[0])));
+      for (int k = 0; k < OUT; ++k) {
+        d[k] = w * inv * (prob[row * OUT + k] - (k == c ? 1.f : 0.f));
+        dz3[row * OUT + k] = d[k];
       }
-      put_split(sD, r, k, v);
-    }
-    publish();
-    if (t == 0) {
-      for (int s = 2; s >= 0; --s)
-        for (int ks = 0; ks < 8; ++ks) {   // dZ1 (M = rows, N = features of H1, K = features of dZ2)
-          const int b = s == 0 && ks >= 4;
-          tcg::mma_f16(taddr + BW_C1 + 128 * b, tcg::sdesc(aD + s * TILE + ks * 256, 128, 2048),
-                       tcg::sdesc(aW2 + ks * 256, 128, 2048), tcg::idesc_bf16(128, 128), b ? ks > 4 : (s < 2 || ks > 0));
-        }
-      for (int s = 2; s >= 0; --s)
-        for (int ks = 0; ks < 8; ++ks)   // gW2^T (M = features of dZ2, N = features of H1 and the ones, K = rows)
-          tcg::mma_f16(taddr + BW_G2, tcg::sdesc(aD + s * TILE + ks * 4096, 2048, 128),
-                       tcg::sdesc(aH + ks * 4608, 2304, 128), tcg::idesc_bf16(128, 144) | kTA | kTB, s < 2 || ks > 0);
-      tcg::commit(bar);
-    }
-    wait();
-    if (!ok) break;
-    // dZ1 over dZ2
-#pragma unroll 1
-    for (int k = 32 * qd; k < 32 * qd + 32; k += 8) {
-      float z[8], z2[8], v[8];
-      tcg::ld8(lane + BW_C1 + k, z);
-      tcg::ld8(lane + BW_C1 + 128 + k, z2);
-      tcg::wait_ld();
-      const uint4 h = *reinterpret_cast<const uint4*>(sH + boff(r, k, 18));
-      const unsigned hw[4] = {h.x, h.y, h.z, h.w};
-#pragma unroll
-      for (int i = 0; i < 8; ++i) v[i] = masked(hw[i >> 1], i, z[i] + z2[i]);
-      put_split(sD, r, k, v);
-    }
-    // the tile's gW2 and gW3
-    if (qd >= 2) add_cols(BW_G2 + 8 * (qd + 16 - 18), 0, sum[4]);
-#pragma unroll
-    for (int i = 5; i < 9; ++i) add_cols(BW_G2 + 8 * (qd + 4 * i - 18), 0, sum[i]);
-    if (qd < 2) add_cols(BW_G3 + 8 * qd, 0, sum[9]);
-    publish();
-    if (t == 0) {
-      for (int s = 2; s >= 0; --s)
-        for (int ks = 0; ks < 8; ++ks) {   // gW1^T (M = features of dZ1, N = inputs and the ones, K = rows)
-          const int b = s == 0 && ks >= 4;
-          tcg::mma_f16(taddr + BW_G1 + 144 * b, tcg::sdesc(aD + s * TILE + ks * 4096, 2048, 128),
-                       tcg::sdesc(aX + ks * 4608, 2304, 128), tcg::idesc_bf16(128, 144) | kTA | kTB,
-                       b ? ks > 4 : (s < 2 || ks > 0));
-        }
-      tcg::commit(bar);
-    }
-    wait();   // the next tile overwrites the operands
-    if (!ok) break;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) add_cols(BW_G1 + 8 * (qd + 4 * i), 144, sum[i]);
-    if (qd < 2) add_cols(BW_G1 + 8 * (qd + 16), 144, sum[4]);
-  }
-  // this CTA's sums, in the parameters' layout
-  if (ok) {
-    float* G = part + (size_t)blockIdx.x * NPARAM;
-#pragma unroll
-    for (int i = 0; i < BW_SUMS; ++i) {
-      const int g = qd + 4 * i;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const float v = sum[i][j];
-        if (g < 18) {
-          const int k = 8 * g + j;
-          if (k < IN) G[OFF_W1 + k * HID + r] = v;
-          else if (k == IN) G[OFF_B1 + r] = v;
-        } else if (g < 36) {
-          const int k = 8 * (g - 18) + j;
-          if (k < HID) G[OFF_W2 + k * HID + r] = v;
-          else if (k == HID) G[OFF_B2 + r] = v;
-        }
-      }
-    }
-    // gW3: the three parts' columns c + 3 s lie in two threads' groups (g = 36,
-    // 37); the ninth column passes through shared memory
-    __syncthreads();
-    if (qd == 1) reinterpret_cast<float*>(sX)[r] = sum[9][0];
-    __syncthreads();
-    if (qd == 0) {
-      const float last = reinterpret_cast<float*>(sX)[r];
-#pragma unroll
-      for (int k = 0; k < OUT; ++k)
-        G[OFF_W3 + r * OUT + k] = sum[9][k] + (sum[9][k + 3] + (k + 6 < 8 ? sum[9][(k + 6) & 7] : last));
+      if (want_loss) loss = (double)w * -log((double)prob[row * OUT + c]);
     }
 #pragma unroll
-    for (int k = 0; k < OUT; ++k) {
-      float v = qd == 0 ? gb3[k] : 0.f;
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if ((t & 31) == 0) sRed[warp * 8 + k] = v;
-    }
+    for (int k = 0; k < OUT; ++k) sD3[t * 4 + k] = d[k];
     if (want_loss) {
       for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
-      if ((t & 31) == 0 && qd == 0) atomicAdd(acc, loss);
+      if ((t & 31) == 0) atomicAdd(acc, loss);
     }
-    __syncthreads();
-    if (t < OUT) G[OFF_B3 + t] = ((sRed[t] + sRed[8 + t]) + sRed[16 + t]) + sRed[24 + t];
-  } else if (!ok && t == 0) {
-    atomicOr(err, 4);
   }
-  tcg::fence_before();
   __syncthreads();
-  if (warp == 0) tcg::dealloc(taddr, 512);
+  // dZ2, 8 features of a row at a time
+  for (int u = t; u < BR_ROWS * (HID / 8); u += BR_T) {
+    const int r = u & (BR_ROWS - 1), k = 8 * (u / BR_ROWS);
+    const long long row = row0 + r;
+    uint4 h = make_uint4(0u, 0u, 0u, 0u);
+    if (row < n) h = *reinterpret_cast<const uint4*>(H2 + row * HID + k);
+    const unsigned hw[4] = {h.x, h.y, h.z, h.w};
+    const float d0 = sD3[r * 4], d1 = sD3[r * 4 + 1], d2 = sD3[r * 4 + 2];
+    float v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const float* w = sW3 + (k + i) * OUT;
+      v[i] = masked(hw[i >> 1], i, fmaf(d2, w[2], fmaf(d1, w[1], d0 * w[0])));
+      sA[(k + i) * (BR_ROWS + 4) + r] = v[i];
+    }
+    if (row < n) {
+      float4* o = reinterpret_cast<float4*>(dz2 + row * HID + k);
+      o[0] = make_float4(v[0], v[1], v[2], v[3]);
+      o[1] = make_float4(v[4], v[5], v[6], v[7]);
+    }
+  }
+  __syncthreads();
+  // dZ1: thread (rows 4 ty.. and 32 + 4 ty.., features 4 tx.. and 64 + 4 tx..),
+  // terms in the order of the features of dZ2
+  const int tx = t & 15, ty = t >> 4;
+  float2 c[8][4];
+#pragma unroll
+  for (int a = 0; a < 8; ++a)
+#pragma unroll
+    for (int b = 0; b < 4; ++b) c[a][b] = make_float2(0.f, 0.f);
+#pragma unroll 4
+  for (int j = 0; j < HID; ++j) {
+    const float4 x = *reinterpret_cast<const float4*>(sA + j * (BR_ROWS + 4) + 4 * ty);
+    const float4 z = *reinterpret_cast<const float4*>(sA + j * (BR_ROWS + 4) + 32 + 4 * ty);
+    const float4 p = *reinterpret_cast<const float4*>(sW + j * BR_LD + 4 * tx);
+    const float4 q = *reinterpret_cast<const float4*>(sW + j * BR_LD + 64 + 4 * tx);
+    const float xs[8] = {x.x, x.y, x.z, x.w, z.x, z.y, z.z, z.w};
+    const float2 w[4] = {make_float2(p.x, p.y), make_float2(p.z, p.w), make_float2(q.x, q.y), make_float2(q.z, q.w)};
+#pragma unroll
+    for (int a = 0; a < 8; ++a)
+#pragma unroll
+      for (int b = 0; b < 4; ++b) c[a][b] = __ffma2_rn(make_float2(xs[a], xs[a]), w[b], c[a][b]);
+  }
+#pragma unroll
+  for (int a = 0; a < 8; ++a) {
+    const long long row = row0 + (a >> 2) * 32 + 4 * ty + (a & 3);
+    if (row >= n) continue;
+#pragma unroll
+    for (int g = 0; g < 2; ++g) {
+      const uint2 h = *reinterpret_cast<const uint2*>(H1 + row * HID + 64 * g + 4 * tx);
+      *reinterpret_cast<float4*>(dz1 + row * HID + 64 * g + 4 * tx) =
+          make_float4(masked(h.x, 0, c[a][2 * g].x), masked(h.x, 1, c[a][2 * g].y), masked(h.y, 0, c[a][2 * g + 1].x),
+                      masked(h.y, 1, c[a][2 * g + 1].y));
+    }
+  }
 }
 
-// gradients: the CTAs' sums, in four groups of consecutive CTAs, added in order
-__global__ void __launch_bounds__(256) mlp_sum(const float* __restrict__ part, int parts, float* __restrict__ G) {
-  __shared__ float sg[4][64];
-  const int l = threadIdx.x & 63, g = threadIdx.x >> 6, i = blockIdx.x * 64 + l;
-  const int per = (parts + 3) / 4, k1 = min(parts, (g + 1) * per);
-  float s = 0.f;
-  if (i < NPARAM) {
-#pragma unroll 8
-    for (int k = g * per; k < k1; ++k) s += part[(size_t)k * NPARAM + i];
-  }
-  sg[g][l] = s;
+// One 64 x 64 block of a weight gradient over one split of the rows: blockIdx.y
+// selects gW1 (inputs x dZ1) or gW2 (H1 x dZ2) and the block of 2 x 2; gW1's
+// blocks have 68 rows, the last four spread over all threads.  A thread owns
+// 4 x 8 gradients; four warps per scheduler cover the loads of the next 32 rows
+// (8 x 8 per thread, half the warps: 225 us against 144 us).
+constexpr int BG_K = 32, BG_T = 128;
+constexpr int PSTRIDE = (NPARAM + 3) / 4 * 4;   // a split's sums: 16-byte aligned rows
+static_assert(OFF_W1 % 4 == 0 && OFF_W2 % 4 == 0, "weight blocks are stored 16 bytes at a time");
+template <int WHICH>
+__device__ __forceinline__ void grad_block(const float* __restrict__ X, const __nv_bfloat16* __restrict__ H1,
+                                           const float* __restrict__ Z, int n, int chunk, int mb, int nb,
+                                           float* __restrict__ part, float (*sA)[BG_K][72], float (*sB)[BG_K][64]) {
+  constexpr int MT = WHICH == 0 ? 68 : 64, QA = MT / 4, NA = (BG_K * QA + BG_T - 1) / BG_T;
+  const int t = threadIdx.x, tx = t & 7, ty = t >> 3, m0 = mb * MT;
+  const long long k0 = (long long)blockIdx.x * chunk, k1 = min((long long)n, k0 + chunk);
+  float4 ra[NA], rb[BG_K * 16 / BG_T];
+  auto load = [&](long long kb) {
+#pragma unroll
+    for (int i = 0; i < NA; ++i) {
+      const int u = t + i * BG_T, r = u / QA, m = 4 * (u - r * QA);
+      ra[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (u < BG_K * QA && kb + r < k1) {
+        if (WHICH == 0) {
+          const float* p = X + (kb + r) * IN + m0 + m;
+          ra[i] = make_float4(bf16r(__ldg(p)), bf16r(__ldg(p + 1)), bf16r(__ldg(p + 2)), bf16r(__ldg(p + 3)));
+        } else {
+          const uint2 h = __ldg(reinterpret_cast<const uint2*>(H1 + (kb + r) * HID + m0 + m));
+          const float2 lo = bf2(h.x), hi = bf2(h.y);
+          ra[i] = make_float4(lo.x, lo.y, hi.x, hi.y);
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < BG_K * 16 / BG_T; ++i) {
+      const int u = t + i * BG_T, r = u >> 4, c = 4 * (u & 15);
+      rb[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (kb + r < k1) rb[i] = __ldg(reinterpret_cast<const float4*>(Z + (kb + r) * HID + nb * 64 + c));
+    }
+  };
+  auto store = [&](int buf) {
+#pragma unroll
+    for (int i = 0; i < NA; ++i) {
+      const int u = t + i * BG_T, r = u / QA, m = 4 * (u - r * QA);
+      if (u < BG_K * QA) *reinterpret_cast<float4*>(&sA[buf][r][m]) = ra[i];
+    }
+#pragma unroll
+    for (int i = 0; i < BG_K * 16 / BG_T; ++i) {
+      const int u = t + i * BG_T;
+      *reinterpret_cast<float4*>(&sB[buf][u >> 4][4 * (u & 15)]) = rb[i];
+    }
+  };
+  // rows 4 ty..; columns 4 tx.., 32 + 4 tx..; rows 64, 65 (66, 67 for t >= 64) of column t mod 64
+  float2 c[4][4], e = make_float2(0.f, 0.f);
+  const int et = t & 63, er = 64 + 2 * (t >> 6);
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < 4; ++b) c[a][b] = make_float2(0.f, 0.f);
+  load(k0);
+  store(0);
   __syncthreads();
-  if (g == 0 && i < NPARAM) G[i] = ((sg[0][l] + sg[1][l]) + sg[2][l]) + sg[3][l];
+  int buf = 0;
+  for (long long kb = k0; kb < k1; kb += BG_K, buf ^= 1) {
+    const bool more = kb + BG_K < k1;
+    if (more) load(kb + BG_K);
+#pragma unroll 8
+    for (int k = 0; k < BG_K; ++k) {
+      const float4 x = *reinterpret_cast<const float4*>(&sA[buf][k][4 * ty]);
+      const float4 p = *reinterpret_cast<const float4*>(&sB[buf][k][4 * tx]);
+      const float4 q = *reinterpret_cast<const float4*>(&sB[buf][k][32 + 4 * tx]);
+      const float xs[4] = {x.x, x.y, x.z, x.w};
+      const float2 w[4] = {make_float2(p.x, p.y), make_float2(p.z, p.w), make_float2(q.x, q.y), make_float2(q.z, q.w)};
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) c[a][b] = __ffma2_rn(make_float2(xs[a], xs[a]), w[b], c[a][b]);
+      if (WHICH == 0) {
+        const float wz = sB[buf][k][et];
+        e = __ffma2_rn(*reinterpret_cast<const float2*>(&sA[buf][k][er]), make_float2(wz, wz), e);
+      }
+    }
+    if (more) store(buf ^ 1);
+    __syncthreads();
+  }
+  float* G = part + (size_t)blockIdx.x * PSTRIDE + (WHICH == 0 ? OFF_W1 : OFF_W2) + (size_t)m0 * HID + nb * 64;
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int g = 0; g < 2; ++g)
+      *reinterpret_cast<float4*>(G + (4 * ty + a) * HID + 32 * g + 4 * tx) =
+          make_float4(c[a][2 * g].x, c[a][2 * g].y, c[a][2 * g + 1].x, c[a][2 * g + 1].y);
+  if (WHICH == 0) {
+    G[er * HID + et] = e.x;
+    G[(er + 1) * HID + et] = e.y;
+  }
+}
+__global__ void __launch_bounds__(BG_T)
+back_grads(const float* __restrict__ X, const __nv_bfloat16* __restrict__ H1, const float* __restrict__ dz1,
+           const float* __restrict__ dz2, int n, int chunk, float* __restrict__ part) {
+  __shared__ __align__(16) float sA[2][BG_K][72], sB[2][BG_K][64];
+  const int mb = (blockIdx.y >> 1) & 1, nb = blockIdx.y & 1;
+  if (blockIdx.y < 4) grad_block<0>(X, H1, dz1, n, chunk, mb, nb, part, sA, sB);
+  else grad_block<1>(X, H1, dz2, n, chunk, mb, nb, part, sA, sB);
+}
+
+// gW3 over the splits' rows and the bias gradients over chunks of 1024 rows:
+// serial sums over the rows of 32 columns per CTA.  Eight warps load 128 rows at
+// a time (16 independent loads per thread), the first one adds them up from
+// shared memory while the others load the next 128.
+constexpr int BT_T = 256, BT_S = 128;
+__global__ void __launch_bounds__(BT_T)
+back_tail(const __nv_bfloat16* __restrict__ H2, const float* __restrict__ dz1, const float* __restrict__ dz2,
+          const float* __restrict__ dz3, int n, int chunk, int splits, float* __restrict__ part,
+          float* __restrict__ bpart) {
+  __shared__ __align__(16) float sV[2][BT_S][32], sD[2][BT_S][4];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool w3 = (int)blockIdx.x < 4 * splits;
+  // bias: 4 CTAs for dZ1, 4 for dZ2 and one for dZ3 per chunk
+  const int u = w3 ? (int)blockIdx.x : (int)blockIdx.x - 4 * splits, ch = w3 ? u >> 2 : u / 9, sl = w3 ? u & 3 : u - 9 * ch;
+  const int len = w3 ? chunk : 1024, cols = !w3 && sl == 8 ? OUT : HID, col = (sl & 3) * 32 + lane;
+  const float* Z = sl < 4 ? dz1 : (sl < 8 ? dz2 : dz3);
+  const long long r0 = (long long)ch * len, r1 = min((long long)n, r0 + len);
+  const bool in = cols == HID || lane < OUT;
+  auto stage = [&](int buf, long long rb) {
+    float v[BT_S / 8];
+#pragma unroll
+    for (int i = 0; i < BT_S / 8; ++i) {
+      const long long r = rb + warp + 8 * i;
+      v[i] = 0.f;
+      if (r < r1 && in) v[i] = w3 ? __bfloat162float(H2[r * HID + col]) : __ldg(Z + r * cols + (cols == HID ? col : lane));
+    }
+    if (w3 && threadIdx.x < BT_S) {
+      const long long r = rb + threadIdx.x;
+#pragma unroll
+      for (int j = 0; j < OUT; ++j) sD[buf][threadIdx.x][j] = r < r1 ? __ldg(dz3 + r * OUT + j) : 0.f;
+    }
+#pragma unroll
+    for (int i = 0; i < BT_S / 8; ++i) sV[buf][warp + 8 * i][lane] = v[i];
+  };
+  float g[3] = {0.f, 0.f, 0.f};
+  stage(0, r0);
+  __syncthreads();
+  int buf = 0;
+  for (long long rb = r0; rb < r1; rb += BT_S, buf ^= 1) {
+    if (warp == 0) {
+      if (w3) {
+#pragma unroll 8
+        for (int i = 0; i < BT_S; ++i) {
+          const float h = sV[buf][i][lane];
+          const float4 d = *reinterpret_cast<const float4*>(sD[buf][i]);
+          g[0] = fmaf(h, d.x, g[0]);
+          g[1] = fmaf(h, d.y, g[1]);
+          g[2] = fmaf(h, d.z, g[2]);
+        }
+      } else {
+#pragma unroll 16
+        for (int i = 0; i < BT_S; ++i) g[0] += sV[buf][i][lane];
+      }
+    }
+    if (rb + BT_S < r1) stage(buf ^ 1, rb + BT_S);
+    __syncthreads();
+  }
+  if (warp != 0) return;
+  if (w3) {
+#pragma unroll
+    for (int j = 0; j < OUT; ++j) part[(size_t)ch * PSTRIDE + OFF_W3 + col * OUT + j] = g[j];
+  } else if (in) {
+    bpart[(size_t)ch * 260 + (sl < 8 ? sl * 32 : 2 * HID) + lane] = g[0];
+  }
+}
+
+// gradients: the splits' (and chunks') sums added in order
+__global__ void __launch_bounds__(128) back_sum(const float* __restrict__ part, int splits, const float* __restrict__ bpart,
+                                                int bchunks, float* __restrict__ G) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= NPARAM) return;
+  const int b = (i >= OFF_B1 && i < OFF_W2) ? i - OFF_B1
+                : ((i >= OFF_B2 && i < OFF_W3) ? HID + i - OFF_B2 : (i >= OFF_B3 ? 2 * HID + i - OFF_B3 : -1));
+  const float* p = b >= 0 ? bpart + b : part + i;
+  const size_t ld = b >= 0 ? 260 : PSTRIDE;
+  const int m = b >= 0 ? bchunks : splits;
+  float s = 0.f;
+#pragma unroll 16
+  for (int k = 0; k < m; ++k) s += p[(size_t)k * ld];
+  G[i] = s;
 }
 
 __global__ void adam_kernel(float* __restrict__ P, const float* __restrict__ G, float* __restrict__ m,
@@ -919,8 +925,8 @@ struct MlpImpl {
   __nv_bfloat16* wt = nullptr;  // transposed bfloat16 weights (W1T | W2T | W3T)
   int max_rows = 0;
   __nv_bfloat16 *H1 = nullptr, *H2 = nullptr;   // hidden activations of the backward pass's forward
-  float *prob = nullptr, *part = nullptr;       // part: the backward CTAs' sums, [ctas][NPARAM]
-  int ctas = 0;
+  float *prob = nullptr, *dz3 = nullptr, *dz2 = nullptr, *dz1 = nullptr;
+  float *part = nullptr, *bpart = nullptr;      // splits' weight gradients [64][PSTRIDE], chunks' bias sums [..][260]
   double* acc = nullptr;   // loss, weight sum
   int* err = nullptr;      // bit 4: a bounded wait of the tensor-core forward ran out
   int step = 0;
@@ -933,9 +939,6 @@ int mlp_create(unsigned long long seed, int max_rows, void** out) {
   m->max_rows = max_rows;
   cudaGetDevice(&m->dev);
   const size_t rows = (size_t)std::max(max_rows, 1);
-  int nsm = 152;
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, m->dev);
-  m->ctas = (int)std::min<size_t>((rows + 127) / 128, (size_t)nsm);
   cudaError_t e = cudaSuccess;
   auto A = [&](void** p, size_t bytes) { if (e == cudaSuccess) e = cudaMalloc(p, bytes); };
   A((void**)&m->P, NPARAM * 4);
@@ -947,7 +950,11 @@ int mlp_create(unsigned long long seed, int max_rows, void** out) {
   A((void**)&m->H1, rows * HID * 2);
   A((void**)&m->H2, rows * HID * 2);
   A((void**)&m->prob, rows * OUT * 4);
-  A((void**)&m->part, (size_t)m->ctas * NPARAM * 4);
+  A((void**)&m->dz3, rows * OUT * 4);
+  A((void**)&m->dz2, rows * HID * 4);
+  A((void**)&m->dz1, rows * HID * 4);
+  A((void**)&m->part, (size_t)64 * PSTRIDE * 4);
+  A((void**)&m->bpart, ((rows + 1023) / 1024) * 260 * 4);
   A((void**)&m->acc, 2 * sizeof(double));
   A((void**)&m->err, sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(m->err, 0, sizeof(int));
@@ -959,7 +966,7 @@ int mlp_create(unsigned long long seed, int max_rows, void** out) {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(mlp_forward_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(mlp_backward_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BW_SMEM);
+    e = cudaFuncSetAttribute(back_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BR_SMEM);
   if (e == cudaSuccess) {
     // Uniform(-1/sqrt(fan_in), 1/sqrt(fan_in)) weights from splitmix64 of
     // (seed, index), zero biases
@@ -978,7 +985,7 @@ int mlp_create(unsigned long long seed, int max_rows, void** out) {
   }
   if (e != cudaSuccess) {
     std::string msg = cudaGetErrorString(e);
-    void* ps[] = {m->P, m->R, m->G, m->M1, m->M2, m->wt, m->H1, m->H2, m->prob, m->part, m->acc, m->err};
+    void* ps[] = {m->P, m->R, m->G, m->M1, m->M2, m->wt, m->H1, m->H2, m->prob, m->dz3, m->dz2, m->dz1, m->part, m->bpart, m->acc, m->err};
     for (void* p : ps)
       if (p) cudaFree(p);
     delete m;
@@ -993,7 +1000,7 @@ int mlp_create(unsigned long long seed, int max_rows, void** out) {
 void mlp_destroy(void* h) {
   MlpImpl* m = (MlpImpl*)h;
   if (!m) return;
-  void* ps[] = {m->P, m->R, m->G, m->M1, m->M2, m->wt, m->H1, m->H2, m->prob, m->part, m->acc, m->err};
+  void* ps[] = {m->P, m->R, m->G, m->M1, m->M2, m->wt, m->H1, m->H2, m->prob, m->dz3, m->dz2, m->dz1, m->part, m->bpart, m->acc, m->err};
   for (void* p : ps)
     if (p) cudaFree(p);
   delete m;
@@ -1067,10 +1074,14 @@ int mlp_backward_api(void* h, const float* X, const int8_t* y, const float* cw, 
   SEM_CUDA_TRY(cudaMemsetAsync(m->acc, 0, 2 * sizeof(double), st));
   mlp_wsum<<<std::min(256, (n + 255) / 256), 256, 0, st>>>(y, n, cw[0], cw[1], cw[2], m->acc);
   ProfScope ps("mlp_backward", st);
-  const int ctas = std::min((n + 127) / 128, m->ctas);
-  mlp_backward_tc<<<ctas, BW_T, BW_SMEM, st>>>(X, y, n, cw[0], cw[1], cw[2], m->prob, m->H1, m->H2, m->R, m->acc,
-                                               loss_host != nullptr, m->part, m->err);
-  mlp_sum<<<(NPARAM + 63) / 64, 256, 0, st>>>(m->part, ctas, m->G);
+  back_rows<<<(n + BR_ROWS - 1) / BR_ROWS, BR_T, BR_SMEM, st>>>(y, n, cw[0], cw[1], cw[2], m->prob, m->H1, m->H2,
+                                                               m->wt + W1T_SZ, m->R, m->acc, loss_host != nullptr, m->dz3, m->dz2, m->dz1);
+  int chunk = 0;
+  const int splits = back_splits(n, chunk), bchunks = (n + 1023) / 1024;
+  back_grads<<<dim3(splits, 8), BG_T, 0, st>>>(X, m->H1, m->dz1, m->dz2, n, chunk, m->part);
+  back_tail<<<4 * splits + 9 * bchunks, BT_T, 0, st>>>(m->H2, m->dz1, m->dz2, m->dz3, n, chunk, splits, m->part,
+                                                       m->bpart);
+  back_sum<<<(NPARAM + 127) / 128, 128, 0, st>>>(m->part, splits, m->bpart, bchunks, m->G);
   SEM_CUDA_TRY(cudaGetLastError());
   if (loss_host) {
     double a[2];
