@@ -113,7 +113,8 @@ def test_speed_criterion_bits(sem, N, nz, eqset):
         np.testing.assert_array_equal(flags.cpu().numpy(), np.where(up, 1, np.where(down, -1, 0)), err_msg=name)
 
 
-@pytest.mark.parametrize("N,nz,n,half", [(4, 3, 4, 40e3), (4, 100, 3, 150e3), (3, 5, 9, 75e3), (6, 1, 4, 10e3)])
+@pytest.mark.parametrize("N,nz,n,half", [(4, 3, 4, 40e3), (4, 100, 3, 150e3), (3, 5, 9, 75e3), (6, 1, 4, 10e3), (2, 3, 40, 60e3),
+                                         (4, 100, 18, 20e3), (3, 11, 24, 150e3)])
 def test_diag_levels(sem, N, nz, n, half):
     """Levels within, across and beyond one block of threads; the node list
     across several blocks."""
