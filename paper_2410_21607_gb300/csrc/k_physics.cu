@@ -21,13 +21,15 @@
 //     the result into r_C[column][ab][field][kz].
 //
 // R is the arithmetic type: double for the float64 form, float for the mixed
-// form (float32 mirror of the state, float32 residuals).  The mixed form of
-// the conservative set uses physics_lines (below) instead, and only for what
-// the element kernel has not added: a line-exchange element kernel adds the
-// absorbing layer, and at order 4 the stress as well (k_stage.cu), in which
-// case this pass runs for the heating alone, if at all.
+// form (float32 mirror of the state, float32 residuals).  The mixed form on box
+// meshes uses physics_lines (below) instead (the paper's set, 40x36x12, N = 4:
+// 107 us as a column kernel), for the conservative set only for what the element
+// kernel has not added: a line-exchange element kernel adds the absorbing layer,
+// and at order 4 the stress as well (k_stage.cu), in which case this pass runs
+// for the heating alone, if at all.
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 #include <vector>
 
 #include "sem_internal.h"
@@ -337,18 +339,20 @@ physics_column(const PhysArgs A) {
 template <int N, typename R>
 void launch_n(const PhysArgs& A, int eq, int ncol, cudaStream_t st) {
   constexpr int threads = ((N + 1) * (N + 1) * (N + 1) + 31) / 32 * 32;
-  if (A.metric) {
-    if (eq == SEM_EQ_CONSERVATIVE) physics_column<N, 0, R, true><<<ncol, threads, 0, st>>>(A);
-    else physics_column<N, 1, R, true><<<ncol, threads, 0, st>>>(A);
-  } else if (eq == SEM_EQ_CONSERVATIVE) {
-    physics_column<N, 0, R><<<ncol, threads, 0, st>>>(A);
-  } else {
-    physics_column<N, 1, R><<<ncol, threads, 0, st>>>(A);
+  if constexpr (std::is_same<R, double>::value) {   // box meshes; the mixed form's take physics_lines
+    if (!A.metric) {
+      if (eq == SEM_EQ_CONSERVATIVE) physics_column<N, 0, R><<<ncol, threads, 0, st>>>(A);
+      else physics_column<N, 1, R><<<ncol, threads, 0, st>>>(A);
+      return;
+    }
   }
+  if (eq == SEM_EQ_CONSERVATIVE) physics_column<N, 0, R, true><<<ncol, threads, 0, st>>>(A);
+  else physics_column<N, 1, R, true><<<ncol, threads, 0, st>>>(A);
 }
 
-// Mixed form, conservative set: the same terms with the thread layout of the
-// line-exchange element kernel (coalesced z-line loads and residual updates).
+// Mixed form, box meshes: the same terms (EQ 0: conservative set, EQ 1: the
+// paper's set, whose velocities are the state and whose stress has no factor
+// rho) with the thread layout of the line-exchange element kernel (coalesced z-line loads and residual updates).
 // Thread (layer kk, line ab) owns the vertical line of N+1 nodes of its
 // element; node (i, j, c) keeps 9 float32 components (u, v, w, then the x and
 // y derivatives, later the weighted x and y stress fluxes) at
@@ -371,7 +375,7 @@ __host__ __device__ constexpr int plines_smem_floats() {
   return KL * plines_ls<N, KL>() + kFields * KL * (N + 1) * (N + 1) + 2 * kFields * (N + 1) * (N + 1);
 }
 
-template <int N, int KL, int MB>
+template <int N, int KL, int MB, int EQ>
 __global__ void __launch_bounds__(KL * (N + 1) * (N + 1), MB)
 physics_lines(const PhysArgs A) {
   constexpr int n1 = N + 1, Nq = n1 * n1;
@@ -441,11 +445,18 @@ physics_lines(const PhysArgs A) {
             for (int f = 0; f < kFields; ++f) v[f] = fmaf(wm, __ldg(pq + (long long)f * A.NG), v[f]);
           }
         }
-        rho[c] = __ldg(ref + (long long)kz * kRef + 3) + v[0];
-        const float inv = __frcp_rn(rho[c]);   // = 1 / rho, correctly rounded
-        zV[0 * n1 + c] = v[1] * inv;
-        zV[1 * n1 + c] = v[2] * inv;
-        zV[2 * n1 + c] = v[3] * inv;
+        if constexpr (EQ == 0) {
+          rho[c] = __ldg(ref + (long long)kz * kRef + 3) + v[0];
+          const float inv = __frcp_rn(rho[c]);   // = 1 / rho, correctly rounded
+          zV[0 * n1 + c] = v[1] * inv;
+          zV[1 * n1 + c] = v[2] * inv;
+          zV[2 * n1 + c] = v[3] * inv;
+        } else {
+          rho[c] = 1.f;
+          zV[0 * n1 + c] = v[1];
+          zV[1 * n1 + c] = v[2];
+          zV[2 * n1 + c] = v[3];
+        }
         if (spg) {
           const float wJ = wi * wj * p_wf[N][c] * J;
           const float Rz = __ldg(spg + kz);
@@ -593,17 +604,32 @@ physics_lines(const PhysArgs A) {
   }
 }
 
-template <int N, int KL, int MB>
+template <int N, int KL, int MB, int EQ>
 int launch_lines(const PhysArgs& A, int ncol, cudaStream_t st) {
   const size_t sm = sizeof(float) * plines_smem_floats<N, KL>();
   static DeviceOnce attr;
   int rc = device_once(attr, [&] {
-    SEM_CUDA_TRY(cudaFuncSetAttribute(physics_lines<N, KL, MB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    SEM_CUDA_TRY(cudaFuncSetAttribute(physics_lines<N, KL, MB, EQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     return SEM_OK;
   });
   if (rc) return rc;
-  physics_lines<N, KL, MB><<<ncol, KL * (N + 1) * (N + 1), sm, st>>>(A);
+  physics_lines<N, KL, MB, EQ><<<ncol, KL * (N + 1) * (N + 1), sm, st>>>(A);
   return SEM_OK;
+}
+// Layers per CTA at order 4: 8, or 6 where its chunks leave fewer layer slots
+// idle (12 layers: 12 slots instead of 16).
+template <int EQ>
+int launch_lines_n(const PhysArgs& A, int N, int ncol, cudaStream_t st) {
+  switch (N) {
+    case 2: return launch_lines<2, 16, 4, EQ>(A, ncol, st);
+    case 3: return launch_lines<3, 16, 2, EQ>(A, ncol, st);
+    case 4:
+      return (A.nz + 5) / 6 * 6 < (A.nz + 7) / 8 * 8 ? launch_lines<4, 6, 5, EQ>(A, ncol, st)
+                                                      : launch_lines<4, 8, 4, EQ>(A, ncol, st);
+    case 5: return launch_lines<5, 4, 4, EQ>(A, ncol, st);
+    case 6: return launch_lines<6, 4, 2, EQ>(A, ncol, st);
+    default: return fail(SEM_ERR_UNSUPPORTED, "order N not compiled");
+  }
 }
 
 }  // namespace
@@ -687,15 +713,8 @@ int launch_physics(Mesh& m, const sem_params& p, const void* q, bool mixed, void
   }
   ProfScope ps("physics", st);
   const int ncol = (int)m.Ncol();
-  if (mixed && p.eqset == SEM_EQ_CONSERVATIVE && !w) {
-    switch (m.N) {
-      case 2: rc = launch_lines<2, 16, 4>(A, ncol, st); break;
-      case 3: rc = launch_lines<3, 16, 2>(A, ncol, st); break;
-      case 4: rc = launch_lines<4, 8, 4>(A, ncol, st); break;
-      case 5: rc = launch_lines<5, 4, 4>(A, ncol, st); break;
-      case 6: rc = launch_lines<6, 4, 2>(A, ncol, st); break;
-      default: return fail(SEM_ERR_UNSUPPORTED, "order N not compiled");
-    }
+  if (mixed && !w) {
+    rc = p.eqset == SEM_EQ_CONSERVATIVE ? launch_lines_n<0>(A, m.N, ncol, st) : launch_lines_n<1>(A, m.N, ncol, st);
     if (rc) return rc;
     SEM_CUDA_TRY(cudaGetLastError());
     return SEM_OK;
