@@ -2220,18 +2220,40 @@ static const PencilVariant kPencil[] = {
 };
 constexpr int kNumPencil = sizeof(kPencil) / sizeof(kPencil[0]);
 
-// default choice before tuning: the line-exchange variant (kind 1, or 5 for
-// the paper's set) with the most layers per CTA that fit nz (ties: more CTAs
-// per SM), else the fewest layers
-static int pencil_default(int N, int nz, int kind = 1) {
+// Default choice before tuning, among the line-exchange variants (kind 1, or 5
+// for the paper's set).  Box meshes: the least work, counted in layer slots of
+// the chunks a column is cut into (the last chunk's idle layers included) times
+// the variant's cost per slot, relative to the best of its order and set
+// (measured on meshes of 2 to 17 layers that fill the GPU); ties: more CTAs per
+// SM.  Taking the most layers per CTA that fit nz instead cost up to 1.6x (17
+// layers of the paper's set, N = 4: 67 us as chunks of 16, 41 us as chunks of 6;
+// 6 layers of the conservative set 39 us as two chunks of 4, 29 us in one of 8;
+// 12 layers of the paper's set 45 us as two chunks of 8, 37 us as two of 6).
+// Warped layers, whose kernels need more registers, keep to the most layers that
+// fit (210 columns of 16 layers, N = 3: 43 us a step, and 49 us with the variant
+// that wins on box meshes).
+static double slot_cost(const PencilVariant& v) {
+  struct C { int kind, N, KL, MB; double c; };
+  static const C tab[] = {{1, 4, 4, 8, 1.34}, {1, 4, 8, 2, 1.05}, {1, 3, 16, 2, 1.08}, {1, 3, 8, 4, 1.03},
+                          {1, 5, 4, 4, 1.02}, {1, 6, 8, 1, 1.06}, {5, 4, 16, 2, 1.28}};
+  for (const C& t : tab)
+    if (t.kind == v.kind && t.N == v.N && t.KL == v.KL && t.MB == v.MB) return t.c;
+  return 1.0;
+}
+static int pencil_default(int N, int nz, bool warped, int kind = 1) {
   int best = -1;
+  double cost = 0.0;
   for (int v = 0; v < kNumPencil; ++v) {
-    if (kPencil[v].N != N || kPencil[v].kind != kind) continue;
-    if (best < 0) { best = v; continue; }
     const PencilVariant& a = kPencil[v];
-    const PencilVariant& b = kPencil[best];
-    const int fa = a.KL <= nz, fb = b.KL <= nz;
-    if (fa != fb ? fa > fb : (a.KL != b.KL ? (fa ? a.KL > b.KL : a.KL < b.KL) : a.MB > b.MB)) best = v;
+    if (a.N != N || a.kind != kind) continue;
+    const int chunks = (nz + a.KL - 1) / a.KL;
+    // warped: the most layers that fit, else the fewest
+    const double c = warped ? (a.KL <= nz ? -a.KL : a.KL)
+                            : slot_cost(a) * chunks * a.KL;
+    if (best < 0 || c < cost || (c == cost && a.MB > kPencil[best].MB)) {
+      best = v;
+      cost = c;
+    }
   }
   return best;
 }
@@ -2239,9 +2261,9 @@ static int pencil_default(int N, int nz, int kind = 1) {
 static int launch_pencil_n(const VolArgs& A, int N, int nz, cudaStream_t st, int variant = -1,
                            bool smag = false) {
   if (variant < 0 || variant >= kNumPencil || kPencil[variant].N != N || kPencil[variant].kind == 5)
-    variant = pencil_default(N, nz);
+    variant = pencil_default(N, nz, A.metric32 != nullptr);
   // warped layers: the line-exchange kernels only
-  if (A.metric32 && variant >= 0 && kPencil[variant].kind != 1) variant = pencil_default(N, nz);
+  if (A.metric32 && variant >= 0 && kPencil[variant].kind != 1) variant = pencil_default(N, nz, true);
   if (variant < 0) return fail(SEM_ERR_UNSUPPORTED, "order N not compiled");
   if (smag) return kPencil[variant].launch_smag(A, st);
   return kPencil[variant].launch(A, st);
@@ -2251,7 +2273,7 @@ static int launch_pencil_n(const VolArgs& A, int N, int nz, cudaStream_t st, int
 // warped layers.
 static int launch_nc_n(const VolArgs& A, int N, int nz, cudaStream_t st, int variant = -1) {
   if (variant < 0 || variant >= kNumPencil || kPencil[variant].N != N || kPencil[variant].kind != 5)
-    variant = pencil_default(N, nz, 5);
+    variant = pencil_default(N, nz, A.metric32 != nullptr, 5);
   if (variant < 0) return fail(SEM_ERR_UNSUPPORTED, "order N not compiled");
   return kPencil[variant].launch(A, st);
 }
@@ -2265,7 +2287,7 @@ static int element_terms(Mesh& m, const sem_params& p, VolArgs& A, bool& sponge_
   // warped layers: the physics pass adds every term (at each node's height)
   if (p.eqset != SEM_EQ_CONSERVATIVE || m.warped()) return SEM_OK;
   int v = m.pencil_variant;
-  if (v < 0 || v >= kNumPencil || kPencil[v].N != m.N) v = pencil_default(m.N, m.nz);
+  if (v < 0 || v >= kNumPencil || kPencil[v].N != m.N) v = pencil_default(m.N, m.nz, false);
   if (v < 0 || (kPencil[v].kind != 1 && kPencil[v].kind != 4)) return SEM_OK;
   if (p.sponge_gamma > 0.0) {
     const int rc = ensure_sponge(m, p);
