@@ -7,6 +7,8 @@
 //     them with the weak-form derivative matrix (Sec. 3, sum factorisation),
 //     adds the face shared with the layer below (vertical DSS inside the
 //     CTA) and writes the column residual r_C[column][ab][field][kz].
+//   volume_chunk<N> (float64, conservative set, box layers): the same residual
+//     by chunks of layers; volume_lines_* (mixed form): by line exchange.
 //   dss_stage<R>: one thread per global node gathers the horizontal
 //     contributions through Q_h^T (Sec. 3.1, modified DSS), divides by the
 //     lumped mass, applies the rigid-lid condition and fuses the RK stage
@@ -2220,15 +2222,30 @@ static const PencilVariant kPencil[] = {
 };
 constexpr int kNumPencil = sizeof(kPencil) / sizeof(kPencil[0]);
 
+static int sm_count() {
+  int dev = 0, nsm = 152;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  return nsm;
+}
+
 // Default choice before tuning, among the line-exchange variants (kind 1, or 5
-// for the paper's set).  Box meshes: the least work, counted in layer slots of
-// the chunks a column is cut into (the last chunk's idle layers included) times
-// the variant's cost per slot, relative to the best of its order and set
-// (measured on meshes of 2 to 17 layers that fill the GPU); ties: more CTAs per
-// SM.  Taking the most layers per CTA that fit nz instead cost up to 1.6x (17
-// layers of the paper's set, N = 4: 67 us as chunks of 16, 41 us as chunks of 6;
-// 6 layers of the conservative set 39 us as two chunks of 4, 29 us in one of 8;
-// 12 layers of the paper's set 45 us as two chunks of 8, 37 us as two of 6).
+// for the paper's set).  A column's chunks of KL layers follow one another, so a
+// mesh whose z-lines are few per SM is bound by the number of chunks: below 640
+// lines per SM the fewest chunks.  Larger meshes: the least work, counted in
+// layer slots of the chunks (the last one's idle layers included) times the
+// variant's cost per slot, relative to the best of its order and set (measured
+// on meshes of 2 to 17 layers that fill the GPU).  Ties: the least work, then
+// more CTAs per SM.  Microseconds a step, two chunks of 16 against three of 8,
+// 17 layers, by lines per SM: N = 4 58 and 64 (420 lines), 82 and 76 (840), 249 and
+// 212 (3040); N = 3 50 and 56 (540), 85 and 73 (1130); N = 6, 9 layers, two chunks of
+// 8 against three of 4: 77 and 84 (435), 138 and 120 (870).  Against the most layers
+// per CTA that fit nz: 6 layers, N = 4, 47 us as two chunks of 4 and 34 us in one of
+// 8 (8x7 columns), 102 and 85 us (34x32); 17 layers of the paper's set 389 us as
+// chunks of 16 and 247 us as chunks of 6 (34x32).
+// The paper's set: the shared memory of 16 layers, N = 4, leaves one CTA per SM, so
+// the fewest chunks only where every column has an SM (9 layers: 72 columns 47 us as
+// one chunk of 16 and 54 us as two of 8, 154 columns 68 and 65 us).
 // Warped layers, whose kernels need more registers, keep to the most layers that
 // fit (210 columns of 16 layers, N = 3: 43 us a step, and 49 us with the variant
 // that wins on box meshes).
@@ -2240,19 +2257,23 @@ static double slot_cost(const PencilVariant& v) {
     if (t.kind == v.kind && t.N == v.N && t.KL == v.KL && t.MB == v.MB) return t.c;
   return 1.0;
 }
-static int pencil_default(int N, int nz, bool warped, int kind = 1) {
+static int pencil_default(int N, int nz, long long ncol, bool warped, int kind = 1) {
   int best = -1;
-  double cost = 0.0;
+  double cost = 0.0, work = 0.0;
+  const long long nsm = sm_count();
+  const bool few = ncol * nz * (N + 1) * (N + 1) < 640 * nsm && (kind != 5 || ncol <= nsm);
   for (int v = 0; v < kNumPencil; ++v) {
     const PencilVariant& a = kPencil[v];
     if (a.N != N || a.kind != kind) continue;
     const int chunks = (nz + a.KL - 1) / a.KL;
+    const double w = slot_cost(a) * chunks * a.KL;
     // warped: the most layers that fit, else the fewest
-    const double c = warped ? (a.KL <= nz ? -a.KL : a.KL)
-                            : slot_cost(a) * chunks * a.KL;
-    if (best < 0 || c < cost || (c == cost && a.MB > kPencil[best].MB)) {
+    const double c = warped ? (a.KL <= nz ? -a.KL : a.KL) : few ? chunks : w;
+    const double t = warped ? 0.0 : w;
+    if (best < 0 || c < cost || (c == cost && (t < work || (t == work && a.MB > kPencil[best].MB)))) {
       best = v;
       cost = c;
+      work = t;
     }
   }
   return best;
@@ -2261,9 +2282,9 @@ static int pencil_default(int N, int nz, bool warped, int kind = 1) {
 static int launch_pencil_n(const VolArgs& A, int N, int nz, cudaStream_t st, int variant = -1,
                            bool smag = false) {
   if (variant < 0 || variant >= kNumPencil || kPencil[variant].N != N || kPencil[variant].kind == 5)
-    variant = pencil_default(N, nz, A.metric32 != nullptr);
+    variant = pencil_default(N, nz, A.Ncol, A.metric32 != nullptr);
   // warped layers: the line-exchange kernels only
-  if (A.metric32 && variant >= 0 && kPencil[variant].kind != 1) variant = pencil_default(N, nz, true);
+  if (A.metric32 && variant >= 0 && kPencil[variant].kind != 1) variant = pencil_default(N, nz, A.Ncol, true);
   if (variant < 0) return fail(SEM_ERR_UNSUPPORTED, "order N not compiled");
   if (smag) return kPencil[variant].launch_smag(A, st);
   return kPencil[variant].launch(A, st);
@@ -2273,7 +2294,7 @@ static int launch_pencil_n(const VolArgs& A, int N, int nz, cudaStream_t st, int
 // warped layers.
 static int launch_nc_n(const VolArgs& A, int N, int nz, cudaStream_t st, int variant = -1) {
   if (variant < 0 || variant >= kNumPencil || kPencil[variant].N != N || kPencil[variant].kind != 5)
-    variant = pencil_default(N, nz, A.metric32 != nullptr, 5);
+    variant = pencil_default(N, nz, A.Ncol, A.metric32 != nullptr, 5);
   if (variant < 0) return fail(SEM_ERR_UNSUPPORTED, "order N not compiled");
   return kPencil[variant].launch(A, st);
 }
@@ -2287,7 +2308,7 @@ static int element_terms(Mesh& m, const sem_params& p, VolArgs& A, bool& sponge_
   // warped layers: the physics pass adds every term (at each node's height)
   if (p.eqset != SEM_EQ_CONSERVATIVE || m.warped()) return SEM_OK;
   int v = m.pencil_variant;
-  if (v < 0 || v >= kNumPencil || kPencil[v].N != m.N) v = pencil_default(m.N, m.nz, false);
+  if (v < 0 || v >= kNumPencil || kPencil[v].N != m.N) v = pencil_default(m.N, m.nz, m.Ncol(), false);
   if (v < 0 || (kPencil[v].kind != 1 && kPencil[v].kind != 4)) return SEM_OK;
   if (p.sponge_gamma > 0.0) {
     const int rc = ensure_sponge(m, p);
@@ -2372,11 +2393,7 @@ static VolArgs make_vol_args(Mesh& m, const sem_params& p, const void* q, bool m
 }
 
 static int grid_cap(long long work, int per_sm = 8) {
-  int dev = 0, nsm = 152;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  long long blocks = (work + 255) / 256;
-  long long cap = (long long)nsm * per_sm;
+  const long long blocks = (work + 255) / 256, cap = (long long)sm_count() * per_sm;
   return (int)(blocks < cap ? (blocks > 0 ? blocks : 1) : cap);
 }
 
