@@ -2427,7 +2427,15 @@ struct IncArgs {
   int* status;
 };
 
-template <int STAGE, bool WARP = false>
+// FIRST: the loads and stores of d, q and stage 1's q_n32 are marked to be
+// evicted from L2 first.  Each of these values is touched once a stage, while the
+// column residual and the next stage's mirror go from one kernel to the next.
+// What bounds the kernel is HBM; where the residual and the two mirrors fit L2
+// (launch_step_mixed) the marks leave it to them: 32x32x16 elements, N = 4,
+// 26.6 us a stage before and 22.3 with them, the step 173 and 157 us; 40x40x14
+// 38.3 and 33.5 us, the step 251 and 231 us.  On larger meshes neither stays, and
+// the marks cost 0.5 to 1 % (64x64x16: 608 and 612 us a step).
+template <int STAGE, bool WARP = false, bool FIRST = false>
 __device__ __forceinline__ void inc_body(const IncArgs& A, const int gidx, int& bad) {
   const int h = (int)((unsigned)gidx / (unsigned)A.NZ);
   const int kz = gidx - h * A.NZ;
@@ -2439,9 +2447,9 @@ __device__ __forceinline__ void inc_body(const IncArgs& A, const int gidx, int& 
 #pragma unroll
   for (int fl = 0; fl < kFields; ++fl) {
     const long long o = (long long)fl * A.NG + gidx;
-    if (STAGE > 0) dprev[fl] = A.d[o];
-    if (STAGE == 1) q32v[fl] = __ldg(A.q32 + o);
-    if (STAGE == 2) qv[fl] = A.q[o];
+    if (STAGE > 0) dprev[fl] = FIRST ? __ldcs(A.d + o) : A.d[o];
+    if (STAGE == 1) q32v[fl] = FIRST ? __ldcs(A.q32 + o) : __ldg(A.q32 + o);
+    if (STAGE == 2) qv[fl] = FIRST ? __ldcs(A.q + o) : A.q[o];
   }
   // warped layers: the lumped mass per node (it does not factorise)
   const float s = WARP ? A.cdt * __ldg(A.Minv_g + gidx) : A.cdt * (__ldg(A.Minv_h + h) * __ldg(A.Minv_z + kz));
@@ -2476,23 +2484,32 @@ __device__ __forceinline__ void inc_body(const IncArgs& A, const int gidx, int& 
     const float inc = (fl == 3 && lid) ? 0.f : acc[fl] * s;
     const float dn = (STAGE == 0) ? inc : fmaf(A.bcoef, dprev[fl], inc);
     if (STAGE < 2) {
-      A.d[o] = dn;
+      if (FIRST) __stcs(A.d + o, dn);
+      else A.d[o] = dn;
       A.qs32[o] = (STAGE == 0 ? __ldg(A.q32 + o) : q32v[fl]) + dn;
     } else {
       const double qn = qv[fl] + f2d_bits(dn);
-      A.q[o] = qn;
+      if (FIRST) __stcs(A.q + o, qn);
+      else A.q[o] = qn;
       A.q32_out[o] = d2f_bits(qn);
       bad |= nonfinite_bits(qn);
     }
   }
 }
 
-template <int STAGE, bool WARP = false>
+template <int STAGE, bool WARP, bool FIRST>
 __global__ void __launch_bounds__(256) dss_inc(const IncArgs A) {
   int bad = 0;
   for (int gidx = blockIdx.x * blockDim.x + threadIdx.x; gidx < A.NG; gidx += gridDim.x * blockDim.x)
-    inc_body<STAGE, WARP>(A, gidx, bad);
+    inc_body<STAGE, WARP, FIRST>(A, gidx, bad);
   if (STAGE == 2 && __any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(A.status, 1);
+}
+
+template <bool WARP, bool FIRST>
+static void launch_inc(const IncArgs& B, int stage, int blocks, cudaStream_t st) {
+  if (stage == 0) dss_inc<0, WARP, FIRST><<<blocks, 256, 0, st>>>(B);
+  else if (stage == 1) dss_inc<1, WARP, FIRST><<<blocks, 256, 0, st>>>(B);
+  else dss_inc<2, WARP, FIRST><<<blocks, 256, 0, st>>>(B);
 }
 
 int launch_step_mixed(Mesh& m, const sem_params& p, double* q, float* q32, float* work32, double dt,
@@ -2502,6 +2519,11 @@ int launch_step_mixed(Mesh& m, const sem_params& p, double* q, float* q32, float
   DeviceTables& D = *m.dev;
   float* d = work32;
   float* qs32 = work32 + (size_t)kFields * m.NG;
+  // the residual and both mirrors within L2 (see inc_body)
+  int dev = 0, l2 = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev);
+  const bool first = sizeof(float) * kFields * ((size_t)m.Ncol() * m.Nq * m.NZr() + 2 * (size_t)m.NG) <= (size_t)l2;
   for (int stage = 0; stage < 3; ++stage) {
     // element work on the stage state's mirror
     VolArgs A = make_vol_args(m, p, stage == 0 ? (const void*)q32 : (const void*)qs32, true, nullptr);
@@ -2541,16 +2563,15 @@ int launch_step_mixed(Mesh& m, const sem_params& p, double* q, float* q32, float
     B.NZr = m.NZr();
     B.status = D.status;
     ProfScope ps("dss_inc_mixed", st);
-    const int blocks = grid_cap(m.NG, 64);
-    if (B.Minv_g) {
-      if (stage == 0) dss_inc<0, true><<<blocks, 256, 0, st>>>(B);
-      else if (stage == 1) dss_inc<1, true><<<blocks, 256, 0, st>>>(B);
-      else dss_inc<2, true><<<blocks, 256, 0, st>>>(B);
-    } else {
-      if (stage == 0) dss_inc<0><<<blocks, 256, 0, st>>>(B);
-      else if (stage == 1) dss_inc<1><<<blocks, 256, 0, st>>>(B);
-      else dss_inc<2><<<blocks, 256, 0, st>>>(B);
-    }
+    // blocks per SM (4 to 8 of them resident): with the marks 231 us a step of
+    // 40x40x14 elements with 16 and 235 with 40 or 64; on larger meshes 605 us
+    // with 40 and 607 with 64 (64x64x16), 1033 and 1049 (32x32x8 refined twice;
+    // 1052 with 16)
+    const int blocks = grid_cap(m.NG, first ? 16 : 40);
+    if (B.Minv_g)
+      first ? launch_inc<true, true>(B, stage, blocks, st) : launch_inc<true, false>(B, stage, blocks, st);
+    else
+      first ? launch_inc<false, true>(B, stage, blocks, st) : launch_inc<false, false>(B, stage, blocks, st);
     SEM_CUDA_TRY(cudaGetLastError());
   }
   return SEM_OK;
@@ -2978,10 +2999,9 @@ static void batch_enqueue(BatchImpl* b, cudaStream_t st) {
       else
         launch_nc_n(b->h_vol[(stage == 0 ? 0 : n) + k], m.N, m.nz, s2, m.nc_variant);
       const IncArgs& B = b->h_inc[stage * n + k];
-      const int blocks = grid_cap(B.NG, 64);   // as in the single-mesh step
-      if (stage == 0) dss_inc<0><<<blocks, 256, 0, s2>>>(B);
-      else if (stage == 1) dss_inc<1><<<blocks, 256, 0, s2>>>(B);
-      else dss_inc<2><<<blocks, 256, 0, s2>>>(B);
+      // without the marks (instances side by side and one after another share
+      // L2); 12 instances: 879 us a step with 16 blocks per SM, 883 with 40
+      launch_inc<false, false>(B, stage, grid_cap(B.NG, 16), s2);
     }
   }
   // the others: persistent column queue and concatenated increment kernel

@@ -1,6 +1,10 @@
-"""The mixed tendency without tuning, on both sides of the sizes where the choice
-of the element kernel changes (few z-lines per SM, a column per SM), against the
-float64 one."""
+"""The mixed form without tuning.
+
+The mixed step on meshes on both sides of the size from which the column
+residual and the two mirrors no longer fit L2 (the gather's loads and stores are
+marked differently there), box and warped, against the float64 step; and the
+tendency on both sides of the sizes where the choice of the element kernel
+changes (few z-lines per SM, a column per SM), against the float64 one."""
 import numpy as np
 import pytest
 
@@ -22,6 +26,23 @@ def sem():
     build.build()
     from paper_2410_21607_gb300 import sem as s
     return s
+
+
+@pytest.mark.parametrize("warp", [None, (500.0, 2, 3)])
+@pytest.mark.parametrize("nx,ny,nz", [(1, 1, 1), (17, 13, 3), (41, 39, 14), (47, 44, 16)])
+def test_mixed_step_matches_float64(sem, nx, ny, nz, warp):
+    """The increment of the step within 1e-4 (the mixed form's bound)."""
+    m = sem.sem_mesh_create(nx * 75e3, ny * 75e3, LZ, nx, ny, nz, 4, warp=warp)
+    q0 = torch.from_numpy(np.ascontiguousarray(random_state(sem.sem_mesh_coords_host(m).T, LZ, 5))).cuda()
+    ref, w1, w2 = q0.clone(), torch.empty_like(q0), torch.empty_like(q0)
+    sem.sem_step(m, sem.sem_params_default(), ref, w1, w2, 0.25)
+    q, q32 = q0.clone(), torch.empty(q0.shape, dtype=torch.float32, device="cuda")
+    work = torch.empty((10, m.NG), dtype=torch.float32, device="cuda")
+    sem.sem_mirror(m, q, q32)
+    sem.sem_step_mixed(m, sem.sem_params_default(precision=sem.SEM_PREC_MIXED), q, q32, work, 0.25)
+    assert np.all(group_rel_l2(host(q - q0), host(ref - q0)) <= 1e-4)
+    assert torch.equal(q32, sem.sem_mirror(m, q, torch.empty_like(q32)))
+    assert sem.sem_status(m) == 0
 
 
 @pytest.mark.parametrize("eqset", [0, 1])
