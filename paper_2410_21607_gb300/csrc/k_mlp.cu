@@ -778,16 +778,18 @@ __global__ void adam_kernel(float* __restrict__ P, const float* __restrict__ G, 
 // features: the state at the 27 points {-1, 0, 1}^3 of every element
 __constant__ double c_fw[kMaxN + 1][3][kMaxN + 1];   // h_m at -1, 0, 1
 
-// v / s rounded to float32, for a float64 v and a float32 s, on the float32
+// (float)(v / s) for a float64 v and a float32 s, bit for bit, on the float32
 // and integer pipes (a float64 division per value kept the float64 pipe 87 %
 // busy): with the significands m = hi + lo of v (hi its leading 24 bits, lo
-// the next 29 rounded to float32) and t of s, one residual correction of the
-// quotient, q = q0 + (hi - q0 t + lo) / t with the residual exact in an FMA
-// (Markstein), then the exponents.  The correction is below one unit in the
-// last place of q0, so the last addition rounds the quotient to within
-// 0.5 (1 + 2^-20) units.  Quotients below half of float32's smallest value
-// give a signed zero; other results outside 2^-110 .. 2^120, infinities and
-// NaN take the float64 division.
+// the next 29 rounded to float32) and t of s, one residual correction
+// c = (hi - q0 t + lo) / t of the quotient q0 with the residual exact in an
+// FMA (Markstein), q = q0 + c, then the exponents.  c is below three units in
+// the last place of q0 and within 2^-20 of one of its value, so q is the
+// rounded quotient unless what q0 + c leaves over (exact by Fast2Sum) is within
+// 2^-17 of a unit of the midpoint between two float32 numbers; those values
+// (one in 10^5), quotients outside 2^-110 .. 2^120, infinities and NaN take the
+// float64 division.  Quotients below half of float32's smallest value give a
+// signed zero.
 struct Divisor {
   float s, t, rt;   // s, its significand with s's sign in 1 <= |t| < 2, 1 / t
   int e;            // exponent of s; beyond the table's range for a special s
@@ -807,11 +809,15 @@ __device__ __forceinline__ float div_to_f32(double v, const Divisor& D) {
   const int e = (int)((vh >> 20) & 0x7ffu) - 1023 - D.e;   // exponent of v / s, or one above it
   const unsigned sign = vh & 0x80000000u;
   if (e < -153) return __uint_as_float(sign ^ (__float_as_uint(D.t) & 0x80000000u));
-  if (e < -110 || e > 120) return (float)(v / (double)D.s);
   const float hi = __uint_as_float(sign | (127u << 23) | ((vh & 0xfffffu) << 3) | (vl >> 29));
   const float lo = __uint_as_float(__float_as_uint((float)(vl & 0x1fffffffu) * 0x1p-52f) | sign);
   const float q0 = hi * D.rt;
-  const float q = fmaf(fmaf(-q0, D.t, hi) + lo, D.rt, q0);
+  const float c = __fmul_rn(fmaf(-q0, D.t, hi) + lo, D.rt);
+  const float q = q0 + c, left = fabsf((q0 - q) + c);
+  // half a unit of q, a quarter below a power of two
+  const unsigned qb = __float_as_uint(q);
+  const float half = __uint_as_float(qb & 0x7f800000u) * ((qb & 0x7fffffu) ? 0x1p-24f : 0x1p-25f);
+  if (e < -110 || e > 120 || left >= half * (1.f - 0x1p-16f)) return (float)(v / (double)D.s);
   return q * __uint_as_float((unsigned)(e + 127) << 23);
 }
 
