@@ -355,7 +355,7 @@ adapt_speed(const AdaptArgs A, const int ncol, const int cols, const int KL) {
     if (act) {
       const float rho0 = EQ == 0 ? (float)A.ref[(long long)kz * kRef + 3] : 1.f;
       PlaneRange R;
-      bool fits = rho0 > 1e-6f && rho0 < 1e20f;
+      bool fits = rho0 > 1e-6f && rho0 < 1e18f;   // 1 / rho^2 is a normal number up to 9e18
 #pragma unroll 5
       for (int ab = 0; ab < Nq; ++ab) {
         const int hm = hmap[ab];
