@@ -18,6 +18,7 @@
 // float for the mixed form (perturbation arithmetic in float32; reference
 // state and metric terms from float64 tables; stage accumulation in float64).
 #include <algorithm>
+#include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
@@ -107,6 +108,7 @@ struct VolArgs {
   float gf, ff, gammaf;
   float bin[8];         // binomial-series coefficients C(gamma, k), k = 1..7
   double bin64[10];     // ... k = 1..10
+  double bin64_max;     // largest |x| for the float64 series (pow1p_m1_f64)
   double geo[kLev][8];
   float geof[kLev][8];
   const float* ref32;
@@ -184,18 +186,27 @@ __device__ __forceinline__ double recip_f64(double x) {
   const double d = fma(-x, y, 1.0);
   return fma(y, fma(d, d, d), y);
 }
-// (1 + x)^gamma - 1 in float64.  For |x| <= 1/32 (perturbations of a few
-// percent) the binomial series sum_{k=1..10} C(gamma, k) x^k in Horner form,
-// whose first dropped term is below 2^-59 of the result: 10 operations on the
-// float64 pipe, where expm1(gamma log1p(x)), taken beyond, costs about 60.
-__device__ __forceinline__ double pow1p_m1_f64(double x, const double* bin, double gam) {
-  if (fabs(x) <= 0.03125) {
+// (1 + x)^gamma - 1 in float64.  For |x| <= xmax (1/32 for gamma up to 10,
+// perturbations of a few percent) the binomial series
+// sum_{k=1..10} C(gamma, k) x^k in Horner form, whose first dropped term is
+// below 2^-58 of the result (series_range): 10 operations on the float64 pipe,
+// where expm1(gamma log1p(x)), taken beyond, costs about 60.
+__device__ __forceinline__ double pow1p_m1_f64(double x, const double* bin, double xmax, double gam) {
+  if (fabs(x) <= xmax) {
     double s = bin[9];
 #pragma unroll
     for (int k = 8; k >= 0; --k) s = fma(s, x, bin[k]);
     return s * x;
   }
   return expm1(gam * log1p(x));
+}
+// Largest |x|, at most 1/32, for which the series' first dropped term
+// C(gamma, 11) x^11 is below 2^-58 of gamma x, given c10 = C(gamma, 10).  The
+// ratio of specific heats is the caller's: C(gamma, 11) / gamma is 1e-3 at 1.4,
+// but 2e6 at 30, where 1/32 would leave an error of 2^-29.
+static double series_range(double gamma, double c10) {
+  const double c11 = std::fabs(c10 * (gamma - 10.0) / 11.0);
+  return c11 > 0.0 ? std::min(1.0 / 32, std::pow(std::ldexp(gamma, -58) / c11, 0.1)) : 1.0 / 32;
 }
 // Gather the 5 fields of local node (ab, kz) of a column (Q row, Sec. 3.1).
 template <int N, typename R>
@@ -307,7 +318,7 @@ volume_column(const VolArgs A) {
       if (EQ == 0) {
         const R U = v[1], V = v[2], W = v[3], Tp = v[4];
         const R u = U * inv, vv = V * inv, w = W * inv;
-        const R pp = p0 * pow1p_m1_f64(Tp * inv_rt0, A.bin64, gam);
+        const R pp = p0 * pow1p_m1_f64(Tp * inv_rt0, A.bin64, A.bin64_max, gam);
         const R rt = rt0 + Tp;
         const R ax = wj * wc * sx, ay = wi * wc * sy, az = wi * wj * sz;
         if (!WARP) {
@@ -334,7 +345,7 @@ volume_column(const VolArgs A) {
         const R u = v[1], vv = v[2], w = v[3], thp = v[4];
         const R th0 = rf[0];
         const R rtp = rho0 * thp + rp * (th0 + thp);
-        const R pp = p0 * pow1p_m1_f64(rtp * inv_rt0, A.bin64, gam);
+        const R pp = p0 * pow1p_m1_f64(rtp * inv_rt0, A.bin64, A.bin64_max, gam);
         const R ax = wj * wc * sx, ay = wi * wc * sy, az = wi * wj * sz;
         sF[0][t] = rho * u * ax;
         sF[1][t] = rho * vv * ay;
@@ -740,7 +751,7 @@ volume_chunk(const VolArgs A) {
       const double p0 = __ldg(rf + 2), rho0 = __ldg(rf + 3), rt0 = __ldg(rf + 4), irt0 = __ldg(rf + 6);
       const double U = v[1], V = v[2], W = v[3];
       const double inv = recip_f64(rho0 + v[0]);
-      const double pp = p0 * pow1p_m1_f64(v[4] * irt0, A.bin64, A.gamma);
+      const double pp = p0 * pow1p_m1_f64(v[4] * irt0, A.bin64, A.bin64_max, A.gamma);
       const double rt = rt0 + v[4];
       const double ax = sLev[4 * l] * sAb[4 * ab], ay = sLev[4 * l + 1] * sAb[4 * ab + 1], az = sAb[4 * ab + 2];
       const double ux = U * inv * ax, vy = V * inv * ay, wz = W * inv * az;
@@ -2379,6 +2390,7 @@ static VolArgs make_vol_args(Mesh& m, const sem_params& p, const void* q, bool m
       if (k <= 7) A.bin[k - 1] = (float)cb;
     }
     A.bin[7] = 0.f;
+    A.bin64_max = series_range(A.gamma, cb);
   }
   for (int l = 0; l < kLev; ++l) {
     const double hx = m.hx(l), hy = m.hy(l), hz = 1.0;   // per unit layer thickness
