@@ -7,8 +7,8 @@
 //     them with the weak-form derivative matrix (Sec. 3, sum factorisation),
 //     adds the face shared with the layer below (vertical DSS inside the
 //     CTA) and writes the column residual r_C[column][ab][field][kz].
-//   volume_chunk<N> (float64, conservative set, box layers): the same residual
-//     by chunks of layers; volume_lines_* (mixed form): by line exchange.
+//   volume_chunk<N> (float64, conservative set, box layers, orders 2 to 5, not
+//     the thinnest meshes): the same residual by chunks of layers; volume_lines_* (mixed form): by line exchange.
 //   dss_stage<R>: one thread per global node gathers the horizontal
 //     contributions through Q_h^T (Sec. 3.1, modified DSS), divides by the
 //     lumped mass, applies the rigid-lid condition and fuses the RK stage
@@ -680,13 +680,13 @@ __global__ void __launch_bounds__(256) mirror_kernel(const double* q, float* q32
 // and buoyancy are added and the column residual is stored.  Lanes run along z
 // throughout.  The level above a chunk is carried into the next one.
 // 32x32x16, N = 4: 471 us, float64 pipe 81 % busy (1024 columns are 3.4 waves of
-// two CTAs per SM); volume_column, a thread per element node, took 652 us (90 %).
+// two CTAs per SM); volume_column, a thread per element node, takes 526 us (652
+// and 90 % with divisions and expm1 at every node).
 template <int N> struct ChunkCfg;
 template <> struct ChunkCfg<2> { static constexpr int KL = 16; };
 template <> struct ChunkCfg<3> { static constexpr int KL = 8; };
 template <> struct ChunkCfg<4> { static constexpr int KL = 8; };
 template <> struct ChunkCfg<5> { static constexpr int KL = 4; };
-template <> struct ChunkCfg<6> { static constexpr int KL = 2; };
 constexpr int kChunkThreads = 256;
 template <int N> struct ChunkSmem {   // in doubles
   static constexpr int Nq = (N + 1) * (N + 1), KL = ChunkCfg<N>::KL, LD = KL * N + 1;
@@ -877,26 +877,52 @@ static int launch_chunk(const VolArgs& A, cudaStream_t st) {
   return SEM_OK;
 }
 
-// The float64 form's other element kernels (the paper's set, warped layers); the
+static int sm_count() {
+  int dev = 0, nsm = 152;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  return nsm;
+}
+
+// The float64 form's column kernel (either set, box or warped layers); the
 // mixed form runs the line-exchange kernels of the variant table instead.
 template <int N, int EQ>
-static void launch_volume_warp(const VolArgs& A, cudaStream_t st) {
-  constexpr int P = (N + 1) * (N + 1) * (N + 1);
-  ProfScope ps("volume_fp64", st);
-  volume_column<N, EQ, double, true><<<A.Ncol, (P + 31) / 32 * 32, 0, st>>>(A);
-}
-template <int N, int EQ>
 static void launch_volume(const VolArgs& A, cudaStream_t st) {
-  if (A.metric) return launch_volume_warp<N, EQ>(A, st);
   constexpr int P = (N + 1) * (N + 1) * (N + 1);
   ProfScope ps("volume_fp64", st);
-  volume_column<N, EQ, double><<<A.Ncol, (P + 31) / 32 * 32, 0, st>>>(A);
+  if (A.metric)
+    volume_column<N, EQ, double, true><<<A.Ncol, (P + 31) / 32 * 32, 0, st>>>(A);
+  else
+    volume_column<N, EQ, double><<<A.Ncol, (P + 31) / 32 * 32, 0, st>>>(A);
+}
+
+// Layers from which volume_chunk is the faster one of the two (conservative
+// set, box layers).  Its chunk of KL layers costs nearly the same with few of
+// them filled, so thin meshes keep volume_column; so do orders 5 and 6, whose
+// chunks of 4 and 2 layers share few levels and whose planes hold 36 and 49 accumulators a
+// thread, except order 5 with more columns than SMs.  Up to 3 columns per SM
+// the chunks' latency hides behind nothing else and fewer layers suffice.
+// Tendency, chunk and column in units of the column's time, by columns: N = 2,
+// 1 layer 1.06 (9) to 1.7 (1024), 2 layers 0.84 and 1.3, 3 layers 0.71, 1.18 and 0.93
+// (2500); N = 3, 2 layers 0.90 (9), 1.11 (196) and 1.27 (600), 3 layers 0.92 (196), 1.16 (600)
+// and 0.94 (2500); N = 4, 2 layers 1.15 to 1.2, 3 layers 1.00 to 1.13, 4 layers 0.93 to 1.03,
+// 16 layers 0.82 to 0.93; N = 5, 5 to 33 layers 1.21 to 1.01 (9), 6 to 18 layers 0.95 to 1.02
+// (196 to 324); N = 6, 2 to 33 layers 1.43 to 1.23 (9), 1.19 to 0.96 (196 to 1024).
+static int chunk_layers(int N, long long ncol) {
+  const long long nsm = sm_count();
+  switch (N) {
+    case 2: return ncol <= 3 * nsm ? 2 : (ncol > 10 * nsm ? 3 : 4);
+    case 3: return ncol <= nsm ? 2 : (ncol <= 3 * nsm || ncol > 10 * nsm ? 3 : 4);
+    case 4: return 4;
+    default: return ncol > nsm ? 6 : 1 << 30;   // order 5
+  }
 }
 
 template <int N>
 static int launch_volume_fp64(const VolArgs& A, int eq, cudaStream_t st) {
-  if (eq == 0 && !A.metric) return launch_chunk<N>(A, st);
-  if (eq == 0) launch_volume_warp<N, 0>(A, st);
+  if constexpr (N <= 5)
+    if (eq == 0 && !A.metric && A.nz >= chunk_layers(N, A.Ncol)) return launch_chunk<N>(A, st);
+  if (eq == 0) launch_volume<N, 0>(A, st);
   else launch_volume<N, 1>(A, st);
   return SEM_OK;
 }
@@ -2232,13 +2258,6 @@ static const PencilVariant kPencil[] = {
     {5, 4, 3, launch_lines_nc<5, 4, 3>, 5},   {6, 4, 2, launch_lines_nc<6, 4, 2>, 5},
 };
 constexpr int kNumPencil = sizeof(kPencil) / sizeof(kPencil[0]);
-
-static int sm_count() {
-  int dev = 0, nsm = 152;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  return nsm;
-}
 
 // Default choice before tuning, among the line-exchange variants (kind 1, or 5
 // for the paper's set).  A column's chunks of KL layers follow one another, so a
