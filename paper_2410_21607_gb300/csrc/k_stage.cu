@@ -2260,50 +2260,56 @@ static const PencilVariant kPencil[] = {
 constexpr int kNumPencil = sizeof(kPencil) / sizeof(kPencil[0]);
 
 // Default choice before tuning, among the line-exchange variants (kind 1, or 5
-// for the paper's set).  A column's chunks of KL layers follow one another, so a
-// mesh whose z-lines are few per SM is bound by the number of chunks: below 640
-// lines per SM the fewest chunks.  Larger meshes: the least work, counted in
-// layer slots of the chunks (the last one's idle layers included) times the
-// variant's cost per slot, relative to the best of its order and set (measured
-// on meshes of 2 to 17 layers that fill the GPU).  Ties: the least work, then
-// more CTAs per SM.  Microseconds a step, two chunks of 16 against three of 8,
-// 17 layers, by lines per SM: N = 4 58 and 64 (420 lines), 82 and 76 (840), 249 and
-// 212 (3040); N = 3 50 and 56 (540), 85 and 73 (1130); N = 6, 9 layers, two chunks of
-// 8 against three of 4: 77 and 84 (435), 138 and 120 (870).  Against the most layers
-// per CTA that fit nz: 6 layers, N = 4, 47 us as two chunks of 4 and 34 us in one of
-// 8 (8x7 columns), 102 and 85 us (34x32); 17 layers of the paper's set 389 us as
-// chunks of 16 and 247 us as chunks of 6 (34x32).
-// The paper's set: the shared memory of 16 layers, N = 4, leaves one CTA per SM, so
-// the fewest chunks only where every column has an SM (9 layers: 72 columns 47 us as
-// one chunk of 16 and 54 us as two of 8, 154 columns 68 and 65 us).
+// for the paper's set): the least estimated time.  A CTA walks its column's
+// chunks of KL layers one after another.  With r CTAs on an SM a chunk takes
+// L + r KL c, in units of a layer's issue time: L is the chain of loads and
+// barriers that a chunk costs however few CTAs there are (in layers: small
+// orders have short ones of a layer and long ones of L), c the variant's cost
+// per layer slot, idle slots of the last chunk included.  The columns run in
+// waves of MB CTAs per SM, the last one with what is left.  L and c are fitted to
+// all variants' times on 2227 meshes of orders 2 to 6 with 1 to 48 layers and 9 to
+// 4096 columns (the tendency below 1000 columns, the element pass above): there the
+// choice takes 1.002 times the best variant's time on average and 1.10 times at
+// worst, the most layers per CTA that fit nz 1.064 and 1.85 times.  Examples,
+// microseconds an element pass: N = 4, 32 layers, 144 columns: two chunks of 16 14.6,
+// four of 8 18.6; 17 layers, 1296 columns: two of 16 65.9, three of 8 53.1; N = 5, 33 layers,
+// 144 columns: five of 8 31.8, nine of 4 45.4; the paper's set, N = 4, 28 layers,
+// 144 columns: two of 16 18.7, five of 6 24.9.
 // Warped layers, whose kernels need more registers, keep to the most layers that
 // fit (210 columns of 16 layers, N = 3: 43 us a step, and 49 us with the variant
 // that wins on box meshes).
+static double chunk_chain(int kind, int N) {
+  static const double box[kMaxN + 1] = {0, 0, 30, 24, 13, 8, 6};
+  return kind == 5 ? 4.5 : box[N];
+}
 static double slot_cost(const PencilVariant& v) {
   struct C { int kind, N, KL, MB; double c; };
-  static const C tab[] = {{1, 4, 4, 8, 1.34}, {1, 4, 8, 2, 1.05}, {1, 3, 16, 2, 1.08}, {1, 3, 8, 4, 1.03},
-                          {1, 5, 4, 4, 1.02}, {1, 6, 8, 1, 1.06}, {5, 4, 16, 2, 1.28}};
+  static const C tab[] = {{1, 2, 32, 2, 1.15}, {1, 3, 8, 4, 0.95}, {1, 4, 16, 2, 1.02}, {1, 4, 8, 4, 0.90},
+                          {1, 4, 8, 3, 0.88},  {1, 4, 8, 2, 0.88}, {1, 4, 4, 8, 1.97},  {1, 5, 4, 4, 1.18},
+                          {1, 6, 8, 1, 1.10},  {5, 4, 6, 4, 1.07}, {5, 4, 8, 3, 0.90},  {5, 4, 8, 2, 0.80},
+                          {5, 4, 16, 2, 1.02}};
   for (const C& t : tab)
     if (t.kind == v.kind && t.N == v.N && t.KL == v.KL && t.MB == v.MB) return t.c;
   return 1.0;
 }
+static double pencil_time(const PencilVariant& v, int nz, long long ncol, long long nsm) {
+  const double L = chunk_chain(v.kind, v.N), work = v.KL * slot_cost(v);
+  const long long waves = ncol / (nsm * v.MB), left = ncol - waves * nsm * v.MB;
+  const double t = waves * (L + v.MB * work) + (left ? L + (left + nsm - 1) / nsm * work : 0.0);
+  return t * ((nz + v.KL - 1) / v.KL);
+}
 static int pencil_default(int N, int nz, long long ncol, bool warped, int kind = 1) {
   int best = -1;
-  double cost = 0.0, work = 0.0;
+  double cost = 0.0;
   const long long nsm = sm_count();
-  const bool few = ncol * nz * (N + 1) * (N + 1) < 640 * nsm && (kind != 5 || ncol <= nsm);
   for (int v = 0; v < kNumPencil; ++v) {
     const PencilVariant& a = kPencil[v];
     if (a.N != N || a.kind != kind) continue;
-    const int chunks = (nz + a.KL - 1) / a.KL;
-    const double w = slot_cost(a) * chunks * a.KL;
     // warped: the most layers that fit, else the fewest
-    const double c = warped ? (a.KL <= nz ? -a.KL : a.KL) : few ? chunks : w;
-    const double t = warped ? 0.0 : w;
-    if (best < 0 || c < cost || (c == cost && (t < work || (t == work && a.MB > kPencil[best].MB)))) {
+    const double c = warped ? (a.KL <= nz ? -a.KL : a.KL) : pencil_time(a, nz, ncol, nsm);
+    if (best < 0 || c < cost || (c == cost && a.MB > kPencil[best].MB)) {
       best = v;
       cost = c;
-      work = t;
     }
   }
   return best;
