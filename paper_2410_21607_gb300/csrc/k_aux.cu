@@ -9,7 +9,7 @@
 //     with C^l the variable chosen for level l (speed by default; vertical
 //     vorticity or dry Ertel potential vorticity from element-local
 //     derivatives).  adapt_speed<N, EQ> is the same criterion where every level
-//     uses the speed.  The speed is evaluated with explicitly rounded float64
+//     uses the speed (not on small thin meshes).  The speed is evaluated with explicitly rounded float64
 //     operations (sqrt(U U + V V + W W) / rho in that order, no contraction
 //     into FMA) so that the decision is taken in float64 exactly as written.
 //   diag_partial, diag_level: Sec. 4.2 diagnostics per vertical level: maximum
@@ -440,14 +440,19 @@ adapt_speed(const AdaptArgs A, const int ncol, const int cols, const int KL) {
   }
 }
 
+static int sm_count() {
+  int dev = 0, nsm = 152;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  return nsm;
+}
+
 template <int N>
 static void launch_speed(const AdaptArgs& A, int ncol, int eq, cudaStream_t st) {
   // layers per chunk: as many as the block's threads have levels; columns per
   // block: as many as fill it, one where the mesh has too few of them to give
   // every SM two blocks
-  int dev = 0, nsm = 152;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  const int nsm = sm_count();
   const int KL = std::min(A.nz, (kSpeedThreads - 1) / N), LV = KL * N + 1;
   const int chunks = (A.nz + KL - 1) / KL;
   int cols = kSpeedThreads / LV;
@@ -465,10 +470,20 @@ template <int N>
 static void launch_adapt_n(const AdaptArgs& A, int ncol, int eq, cudaStream_t st) {
   constexpr int P = (N + 1) * (N + 1) * (N + 1);
   constexpr int nt = (P + 31) / 32 * 32;
-  // the speed at every level: bounded in float32 first
+  // The speed at every level: bounded in float32 first, except on small thin
+  // meshes.  There a thread's chain over its level's (N+1)^2 nodes (7, 9, 12, 16 and
+  // 20 us for N = 2 to 6, whatever the size) is longer than the general
+  // kernel's, whose threads have a node per layer.  Microseconds, general and speed kernel: one layer, N = 3,
+  // 1024 columns 7.6 and 9.2, 2500 15.5 and 9.1; N = 5, 324 columns 10.9 and 15.8, 600 16.8
+  // and 15.8; two layers, N = 4, 144 columns 7.1 and 12.1, 600 14.8 and 12.2; N = 6, 144 columns
+  // 13.9 and 20.1, 196 21.0 and 20.2; three layers, N = 4, 144 columns 9.9 and 12.1, 196 13.1
+  // and 12.2; N = 2 8.0 and 6.8; four layers, N = 5 17.6 and 16.1.
   bool speed = true;
   for (int k = 0; k < SEM_MAX_THRESHOLDS; ++k) speed = speed && A.var[k] == SEM_CRIT_SPEED;
-  if (speed) return launch_speed<N>(A, ncol, eq, st);
+  const long long nsm = sm_count();
+  const bool thin = A.nz <= 2 ? ncol <= nsm || (long long)ncol * A.nz * std::max(nt, 64) <= 600 * nsm
+                              : A.nz == 3 && N >= 3 && ncol <= nsm;
+  if (speed && !thin) return launch_speed<N>(A, ncol, eq, st);
   if (eq == 0)
     adapt_column<N, 0><<<ncol, nt, 0, st>>>(A);
   else

@@ -46,6 +46,17 @@ def test_speed_kernel_equals_general_kernel(sem, N, nz, eqset, warp):
         np.testing.assert_array_equal(f1, f2, err_msg=name)
 
 
+@pytest.mark.parametrize("N,nz,n", [(2, 1, 54), (2, 2, 28), (2, 3, 4), (3, 1, 40), (3, 2, 28), (3, 3, 13), (4, 1, 28),
+                                    (4, 2, 20), (4, 3, 13), (5, 1, 22), (5, 2, 16), (6, 1, 18), (6, 2, 14), (6, 3, 13)])
+def test_thin_meshes(sem, N, nz, n):
+    """One to three layers where the speed kernel takes over from the general one."""
+    m = make(sem, N, nz, n)
+    for name, q in states(sem, m, 0):
+        (f1, c1), (f2, c2) = both(sem, m, q, thresholds=THR)
+        np.testing.assert_array_equal(c1, c2, err_msg=name)
+        np.testing.assert_array_equal(f1, f2, err_msg=name)
+
+
 def test_density_whose_inverse_square_underflows(sem):
     """1 / rho^2 below float32's normal range: the float32 bounds lose bits there."""
     m = make(sem, 4, 4)
