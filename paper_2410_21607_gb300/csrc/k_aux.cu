@@ -543,24 +543,32 @@ int launch_adapt(Mesh& m, const sem_params& p, const double* q, int8_t* flags, d
 }
 
 // ---------------------------------------------------------------------------
-// Wind diagnostics in two passes.  diag_partial: one CTA per 32 horizontal
-// nodes lists those inside the sub-domain (most CTAs have none and end there)
+// Wind diagnostics in two passes.  diag_partial: one CTA per 8 to 32 horizontal
+// nodes (diag_lines) lists those inside the sub-domain (most CTAs have none and end there)
 // and, lanes along z so that the loads are contiguous, reduces each level over
 // the list, dealt out to as many groups of warps as fit (a node costs a float64
 // root and a divide, in a serial chain per level), the groups' values added in
 // order; diag_level: one CTA per level reduces the CTAs' partial values in a
 // fixed order.  64x64x16, N = 4, 100 km: 28 + 7 us; 135 us as one CTA per level
 // walking all horizontal nodes with loads NZ apart.
-constexpr int kDiagLines = 32, kDiagThreads = 384;
+constexpr int kDiagThreads = 384;
+// Horizontal nodes per CTA of diag_partial.  More levels leave fewer groups, and
+// the nodes of a small sub-domain, which lie side by side, fall on few SMs: with
+// 32 nodes a CTA and 129 levels, 9216 nodes and 100 km took 62 us (48 as one
+// launch), with 8 nodes 48.  On larger meshes the CTAs outside the sub-domain cost
+// more than that: 65536 nodes, 65 levels, 20 km: 38 us with 32.
+static int diag_lines(long long NH, int NZ) {
+  return NZ <= 32 || NH >= 50000 ? 32 : (NH < 20000 ? 8 : 16);
+}
 __global__ void __launch_bounds__(kDiagThreads)
 diag_partial(const double* __restrict__ q, const double* __restrict__ xh, const double* __restrict__ yh,
              const double* __restrict__ Mh, const double* __restrict__ ref, long long NH, int NZ, long long NG,
-             double hw, int eq, const double* __restrict__ refG, const double* __restrict__ Minv_g,
+             double hw, int eq, const double* __restrict__ refG, const double* __restrict__ Minv_g, int lines,
              double* __restrict__ part /*[chunks][NZ][3]*/, int* __restrict__ count) {
-  __shared__ int s_h[kDiagLines];
-  const long long h0 = (long long)blockIdx.x * kDiagLines;
+  __shared__ int s_h[32];
+  const long long h0 = (long long)blockIdx.x * lines;
   const int lane = threadIdx.x & 31;
-  const bool in = h0 + lane < NH && fabs(xh[h0 + lane]) <= hw + 1e-6 && fabs(yh[h0 + lane]) <= hw + 1e-6;
+  const bool in = lane < lines && h0 + lane < NH && fabs(xh[h0 + lane]) <= hw + 1e-6 && fabs(yh[h0 + lane]) <= hw + 1e-6;
   const unsigned mask = __ballot_sync(0xffffffffu, in);
   const int n = __popc(mask);
   if (threadIdx.x == 0) count[blockIdx.x] = n;
@@ -672,25 +680,33 @@ diag_level_small(const double* __restrict__ q, const double* __restrict__ xh, co
 
 // doubles of D.diag_buf: the levels' results, the partial values, the counts
 size_t diag_doubles(const Mesh& m) {
-  const size_t chunks = (size_t)((m.NH + kDiagLines - 1) / kDiagLines);
+  const int lines = diag_lines(m.NH, m.NZ);
+  const size_t chunks = (size_t)((m.NH + lines - 1) / lines);
   return (size_t)m.NZ * 4 + chunks * m.NZ * 3 + (chunks + 1) / 2;
 }
 
 int launch_diag(Mesh& m, const sem_params& p, const double* q, double hw, sem_diag_out* out,
                 cudaStream_t st) {
   DeviceTables& D = *m.dev;
-  const int chunks = (int)((m.NH + kDiagLines - 1) / kDiagLines);
+  const int lines = diag_lines(m.NH, m.NZ), chunks = (int)((m.NH + lines - 1) / lines);
   double* part = D.diag_buf + (size_t)m.NZ * 4;
   int* count = reinterpret_cast<int*>(part + (size_t)chunks * m.NZ * 3);
   const double *refG = m.warped() ? D.refG : nullptr, *Minv_g = m.warped() ? D.Minv_g : nullptr;
-  // up to 16 nodes per thread the single launch is the faster one (a mesh of 300
-  // nodes: 9 us less than the two; 65536 nodes: 135 us against 35)
-  if (m.NH <= 4096) {
+  // One launch up to 4096 nodes (16 per thread), and up to 8192 where about one
+  // node per thread lies in the sub-domain (as if the nodes were spread evenly);
+  // it walks all nodes and costs a root and a divide per 256 inside.  N = 4,
+  // 17 levels, one launch and two: 4624 nodes, 20 km 32 and 35 us, 100 km 44 and 37, all
+  // 60 and 36; 9216 nodes, 20 km 35 and 35; 65536 nodes, 100 km 94 and 46 (with the copy
+  // to the host).  With many levels one launch fills the SMs by itself and stays
+  // the faster one longer (129 levels, 100 km: 6400 nodes 45 and 53, 25600 58 and 53).
+  const long long one = m.NZ > 80 ? std::min(128LL * m.NZ, 16384LL) : 4096;
+  const double inside = (double)m.NH * std::min(1.0, 2.0 * hw / m.Lx) * std::min(1.0, 2.0 * hw / m.Ly);
+  if (m.NH <= one || (m.NH <= 8192 && inside <= 256.0)) {
     diag_level_small<<<m.NZ, 256, 0, st>>>(q, D.xh, D.yh, D.Mh, D.ref, m.NH, m.NZ, m.NG, hw, p.eqset, refG, Minv_g,
                                            D.diag_buf);
   } else {
     diag_partial<<<chunks, kDiagThreads, 0, st>>>(q, D.xh, D.yh, D.Mh, D.ref, m.NH, m.NZ, m.NG, hw, p.eqset, refG,
-                                                  Minv_g, part, count);
+                                                  Minv_g, lines, part, count);
     diag_level<<<m.NZ, 256, 0, st>>>(part, count, chunks, m.NZ, D.diag_buf);
   }
   SEM_CUDA_TRY(cudaGetLastError());

@@ -21,7 +21,8 @@ def sem():
 
 
 @pytest.mark.parametrize("warp", [None, (500.0, 2, 3)])
-@pytest.mark.parametrize("N,nz,nx,ny,half", [(4, 3, 16, 16, 70e3), (4, 3, 17, 17, 70e3), (2, 20, 45, 46, 20e3), (4, 97, 17, 16, 500e3)])
+@pytest.mark.parametrize("N,nz,nx,ny,half", [(4, 3, 16, 16, 70e3), (4, 3, 17, 17, 70e3), (2, 20, 45, 46, 20e3), (4, 97, 17, 16, 500e3),
+                                              (4, 9, 36, 36, 60e3), (2, 3, 112, 112, 100e3), (2, 200, 65, 64, 20e3)])
 def test_diag_levels_at_node_heights(sem, N, nz, nx, ny, half, warp):
     m = sem.sem_mesh_create(300e3, 300e3, LZ, nx, ny, nz, N, warp=warp)
     xyz = sem.sem_mesh_coords_host(m)
