@@ -23,7 +23,7 @@
 // R is the arithmetic type: double for the float64 form, float for the mixed
 // form (float32 mirror of the state, float32 residuals).  The mixed form on box
 // meshes uses physics_lines (below) instead (the paper's set, 40x36x12, N = 4:
-// 107 us as a column kernel), for the conservative set only for what the element
+// 49 us, 107 as a column kernel, which it keeps on thin meshes of orders 2 and 3), for the conservative set only for what the element
 // kernel has not added: a line-exchange element kernel adds the absorbing layer,
 // and at order 4 the stress as well (k_stage.cu), in which case this pass runs
 // for the heating alone, if at all.
@@ -339,12 +339,14 @@ physics_column(const PhysArgs A) {
 template <int N, typename R>
 void launch_n(const PhysArgs& A, int eq, int ncol, cudaStream_t st) {
   constexpr int threads = ((N + 1) * (N + 1) * (N + 1) + 31) / 32 * 32;
-  if constexpr (std::is_same<R, double>::value) {   // box meshes; the mixed form's take physics_lines
-    if (!A.metric) {
-      if (eq == SEM_EQ_CONSERVATIVE) physics_column<N, 0, R><<<ncol, threads, 0, st>>>(A);
-      else physics_column<N, 1, R><<<ncol, threads, 0, st>>>(A);
-      return;
-    }
+  if (!A.metric) {   // box meshes; the mixed form only where lines_pay says so
+    if constexpr (std::is_same<R, double>::value)
+      if (eq == SEM_EQ_CONSERVATIVE) {
+        physics_column<N, 0, R><<<ncol, threads, 0, st>>>(A);
+        return;
+      }
+    if constexpr (std::is_same<R, double>::value || N <= 3) physics_column<N, 1, R><<<ncol, threads, 0, st>>>(A);
+    return;
   }
   if (eq == SEM_EQ_CONSERVATIVE) physics_column<N, 0, R, true><<<ncol, threads, 0, st>>>(A);
   else physics_column<N, 1, R, true><<<ncol, threads, 0, st>>>(A);
@@ -617,16 +619,41 @@ int launch_lines(const PhysArgs& A, int ncol, cudaStream_t st) {
   physics_lines<N, KL, MB, EQ><<<ncol, KL * (N + 1) * (N + 1), sm, st>>>(A);
   return SEM_OK;
 }
+int sm_count() {
+  int dev = 0, nsm = 152;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  return nsm;
+}
+// Whether the paper's set on boxes runs physics_lines: not at orders 2 and 3 with
+// so few layers that most of its 16 layer slots idle, where physics_column does
+// the layers one after another in smaller CTAs.  Microseconds a pass, column and
+// lines: N = 3, 1 layer, 9 columns 8 and 11, 2500 20 and 62; 2 layers, 4096 82 and 82; N = 2,
+// 2 layers, 324 columns 9.8 and 10.2, 2500 12 and 28; 4 layers, 600 13.7 and 12.3, 1024 14.4 and
+// 16.6; 7 layers, 1024 20.5 and 16.2, 2500 26 and 29; 9 layers, 4096 48 and 41.
+bool lines_pay(int N, int nz, int ncol) {
+  if (N == 2) return nz > 7 || (nz > 1 && 4LL * ncol <= 5LL * sm_count() * nz);
+  return N != 3 || nz > 1;
+}
 // Layers per CTA at order 4: 8, or 6 where its chunks leave fewer layer slots
-// idle (12 layers: 12 slots instead of 16).
+// idle (12 layers: 12 slots instead of 16).  In the conservative set the pass is the
+// heating's float64 work; up to a column per SM it is bound by its chain of chunks, and
+// 8 stays where 6 takes more of them or two nearly full ones.  Microseconds, 8 and 6,
+// by layers: 81 columns, 6 33 and 27, 9 43 and 36, 12 43 and 49, 17 70 and 57, 25 79 and 85;
+// 1024 columns, 12 140 and 118, 25 270 and 265.
+bool six_layers(int nz, bool heating, int ncol) {
+  const int c6 = (nz + 5) / 6, c8 = (nz + 7) / 8;
+  if (heating && ncol <= sm_count()) return c6 == c8 && nz != 11 && nz != 12;
+  return c6 * 6 < c8 * 8;
+}
 template <int EQ>
 int launch_lines_n(const PhysArgs& A, int N, int ncol, cudaStream_t st) {
   switch (N) {
     case 2: return launch_lines<2, 16, 4, EQ>(A, ncol, st);
     case 3: return launch_lines<3, 16, 2, EQ>(A, ncol, st);
     case 4:
-      return (A.nz + 5) / 6 * 6 < (A.nz + 7) / 8 * 8 ? launch_lines<4, 6, 5, EQ>(A, ncol, st)
-                                                      : launch_lines<4, 8, 4, EQ>(A, ncol, st);
+      return six_layers(A.nz, EQ == 0, ncol) ? launch_lines<4, 6, 5, EQ>(A, ncol, st)
+                                             : launch_lines<4, 8, 4, EQ>(A, ncol, st);
     case 5: return launch_lines<5, 4, 4, EQ>(A, ncol, st);
     case 6: return launch_lines<6, 4, 2, EQ>(A, ncol, st);
     default: return fail(SEM_ERR_UNSUPPORTED, "order N not compiled");
@@ -714,7 +741,7 @@ int launch_physics(Mesh& m, const sem_params& p, const void* q, bool mixed, void
   }
   ProfScope ps("physics", st);
   const int ncol = (int)m.Ncol();
-  if (mixed && !w) {
+  if (mixed && !w && (p.eqset == SEM_EQ_CONSERVATIVE || lines_pay(m.N, m.nz, ncol))) {
     rc = p.eqset == SEM_EQ_CONSERVATIVE ? launch_lines_n<0>(A, m.N, ncol, st) : launch_lines_n<1>(A, m.N, ncol, st);
     if (rc) return rc;
     SEM_CUDA_TRY(cudaGetLastError());
