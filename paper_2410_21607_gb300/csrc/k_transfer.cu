@@ -116,16 +116,28 @@ struct TrArgs {
 // 468 us, and 147 us for transfer_gather, which moves the unchanged lines
 // itself; 2348 and 204 us when every column was mapped node by node and every
 // value weighted.
+// Values of one field and level on N + 1 lines of a source column.  The loads
+// of all lines are issued before any is looked at (a hanging one's from line 0,
+// then replaced): behind a branch per line they wait for one another, 100 times for a
+// coarsened column of order 4, which thin meshes cannot hide (2 layers, order 4, 64
+// columns: a coarsening 60 us, now 54).
 template <int N>
-__device__ __forceinline__ double old_value(const TrArgs& A, const int hm, const int f, const int kz) {
+__device__ __forceinline__ void old_values(const TrArgs& A, const int* hm, const int f, const int kz, double (&r)[N + 1]) {
   const double* q = A.qold + (long long)f * A.old_NG + kz;
-  if (hm >= 0) return __ldg(q + (long long)hm * A.NZ);
-  const int k = -1 - hm;
-  double v = 0.0;
+  int h[N + 1];
+#pragma unroll
+  for (int m = 0; m <= N; ++m) h[m] = hm[m];
+#pragma unroll
+  for (int m = 0; m <= N; ++m) r[m] = __ldg(q + (long long)max(h[m], 0) * A.NZ);
 #pragma unroll
   for (int m = 0; m <= N; ++m)
-    v += A.old_hang_w[k * (N + 1) + m] * __ldg(q + (long long)A.old_hang_h[k * (N + 1) + m] * A.NZ);
-  return v;
+    if (h[m] < 0) {
+      const int k = -1 - h[m];
+      r[m] = 0.0;
+#pragma unroll
+      for (int n = 0; n <= N; ++n)
+        r[m] += A.old_hang_w[k * (N + 1) + n] * __ldg(q + (long long)A.old_hang_h[k * (N + 1) + n] * A.NZ);
+    }
 }
 // One (field, level) of a new column from its source columns.  The operator
 // tables are indexed directly (not through a selected pointer, which would make
@@ -148,8 +160,7 @@ __device__ __forceinline__ void new_plane(const TrArgs& A, const int* o, const i
 #pragma unroll
       for (int j = 0; j < n1; ++j) {
         double r[n1];
-#pragma unroll
-        for (int m = 0; m < n1; ++m) r[m] = old_value<N>(A, hm[m + n1 * j], f, kz);
+        old_values<N>(A, hm + n1 * j, f, kz, r);
 #pragma unroll
         for (int i = 0; i < n1; ++i)
 #pragma unroll
