@@ -170,11 +170,12 @@ __device__ __forceinline__ const R* ref_row(const VolArgs& A, int hm, int kz) {
   return refH_of<R>(A) + ((long long)(-1 - hm) * A.NZ + kz) * kRef;
 }
 
-// 1 / x of a float64: a float32 reciprocal of x's leading bits (relative error
-// e below 2^-21) and one third-order step y (1 + e + e^2), three fused
-// multiply-adds instead of a float64 division on the narrow float64 pipe; the
-// remaining error is that of the last rounding.  Outside float32's comfortable
-// range the division.
+// 1 / x of a float64: the float32 reciprocal y of x's leading bits, d = 1 - x y
+// exact in a fused multiply-add (|d| below 2^-21), and 1 / x = y / (1 - d) as the
+// geometric series y (1 + d + d^2), the third-order member of Newton's family:
+// three fused multiply-adds instead of a float64 division on the narrow float64
+// pipe.  What the series drops is below 2^-63, so the result is within
+// 0.5 (1 + 2^-9) units.  Outside float32's comfortable range the division.
 __device__ __forceinline__ double recip_f64(double x) {
   const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
   const int e = (int)((hi >> 20) & 0x7ffu) - 1023;
