@@ -171,7 +171,7 @@ __device__ __forceinline__ const R* ref_row(const VolArgs& A, int hm, int kz) {
 }
 
 // 1 / x of a float64: the float32 reciprocal y of x's leading bits, d = 1 - x y
-// exact in a fused multiply-add (|d| below 2^-21), and 1 / x = y / (1 - d) as the
+// in one fused multiply-add (|d| below 2^-21), and 1 / x = y / (1 - d) as the
 // geometric series y (1 + d + d^2), the third-order member of Newton's family:
 // three fused multiply-adds instead of a float64 division on the narrow float64
 // pipe.  What the series drops is below 2^-63, so the result is within
